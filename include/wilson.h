@@ -53,7 +53,12 @@ extern "C" {
  * computes with FP32 instructions (~2^-44 relative rounding per operation);
  * mixed-precision solves use it for their intermediate outer residuals,
  * because GB300 executes FP32 many times faster than FP64.  The final
- * convergence check of every solve is IEEE FP64. */
+ * convergence check of every solve is WL_F64.
+ * WL_F64 fields are IEEE binary64.  The WL_F64 hopping term sums a site's
+ * eight neighbours in 64-bit fixed point (units about 2^-56 of the largest
+ * neighbour component, more accurate than binary64 sums of terms of that size)
+ * when every link entry has a modulus of at most 1.25, as SU(3) links do, and
+ * the neighbours lie between 2^-953 and 2^1007; in binary64 otherwise. */
 typedef enum { WL_F64 = 0, WL_F32 = 1, WL_F16 = 2, WL_DF64 = 3 } wl_prec;
 
 #define WL_PREC_MASK(p) (1 << (p))

@@ -30,6 +30,7 @@ static constexpr int kMaxBatchLat = 64;
 struct BLat {
     Geom g;
     const void* links[2];
+    int fx64;  // links[] are fixed point (FP64 inner iterations only)
     double kappa2;
     int nrhs;
     int item0;   // first hop work item of this lattice
@@ -137,7 +138,12 @@ __global__ void __launch_bounds__(256) batch_hop_kernel(const BatchArgs B)
                     a = -L.kappa2;
                 }
                 cx<T> acc[12];
-                hop_site<P, false>(acc, nb, L.g.Vh, in, smem, kTile, lane);
+                if constexpr (P == WL_F64) {
+                    if (L.fx64) hop_site<P, false, 3>(acc, nb, L.g.Vh, in, smem, kTile, lane);
+                    else hop_site<P, false>(acc, nb, L.g.Vh, in, smem, kTile, lane);
+                } else {
+                    hop_site<P, false>(acc, nb, L.g.Vh, in, smem, kTile, lane);
+                }
                 if (CLOV && L.clov[0]) {
                     if (DOT)
                         epilogue_ptrs<P, DOT, kClX2>(acc, a, nullptr, x1, 1.0, w, out, L.g.Vh, i, part,
@@ -511,6 +517,7 @@ static int batch_context(const std::vector<SolveState>& st, int P, std::shared_p
         L.g = S.g->geo;
         L.links[0] = S.g->links[P][0];
         L.links[1] = S.g->links[P][1];
+        L.fx64 = P == WL_F64 && S.g->fx64;
         L.kappa2 = S.g->kappa * S.g->kappa;
         L.nrhs = S.nrhs;
         L.item0 = item;

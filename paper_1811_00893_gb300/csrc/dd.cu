@@ -20,12 +20,19 @@ extern template struct DDKernels<0, kClX2>;    // dd_hop_clover.cu
 extern template struct DDKernels<0, kClOut>;
 extern template struct DDKernels<1, kClX2>;    // dd_hop_r12_clover.cu
 extern template struct DDKernels<1, kClOut>;
+extern template struct DDKernels<3, kClNone>;  // dd_hop_fx.cu
+extern template struct DDKernels<3, kClX2>;
+extern template struct DDKernels<3, kClOut>;
 
 // the kernel family of a launch: link format and clover mode
 static void dd_hop_family(int lf, int cl, int prec, bool dagger, bool dot, bool bnd, const DDArgs& A, dim3 grid,
                           cudaStream_t s)
 {
-    if (lf) {
+    if (lf == 3) {  // fixed-point FP64 links
+        if (cl == kClX2) DDKernels<3, kClX2>::hop(prec, dagger, dot, bnd, A, grid, s);
+        else if (cl == kClOut) DDKernels<3, kClOut>::hop(prec, dagger, dot, bnd, A, grid, s);
+        else DDKernels<3, kClNone>::hop(prec, dagger, dot, bnd, A, grid, s);
+    } else if (lf) {
         if (cl == kClX2) DDKernels<1, kClX2>::hop(prec, dagger, dot, bnd, A, grid, s);
         else if (cl == kClOut) DDKernels<1, kClOut>::hop(prec, dagger, dot, bnd, A, grid, s);
         else DDKernels<1, kClNone>::hop(prec, dagger, dot, bnd, A, grid, s);
@@ -297,7 +304,9 @@ int dd_launch_hop(wl_dd dd, const DDLaunch& h, cudaStream_t s)
         if (!dd->dom[d]->links[P][0])
             return set_error(WL_ERR_STATE, "domain decomposition was created without the requested precision");
     static const bool r12_off = getenv("WL_NO_R12") != nullptr;
-    const int lf = (P == WL_F32 || P == WL_F16) && dd->dom[0]->links_r12[P][0] && !r12_off ? 1 : 0;
+    const int lf = (P == WL_F32 || P == WL_F16) && dd->dom[0]->links_r12[P][0] && !r12_off ? 1
+                   : P == WL_F64 && dd->dom[0]->fx64                                        ? 3
+                                                                                            : 0;
     const int np = h.nparity, nrhs = h.nrhs;
     const Geom& g = dd->gloc;
 
@@ -341,7 +350,7 @@ int dd_launch_hop(wl_dd dd, const DDLaunch& h, cudaStream_t s)
         wl_gauge gd = dd->dom[d];
         for (int k = 0; k < np; ++k) {
             const int p = h.parity0 + k;
-            D.links[k] = lf ? gd->links_r12[P][p] : gd->links[P][p];
+            D.links[k] = lf == 1 ? gd->links_r12[P][p] : gd->links[P][p];
             D.in[k] = (const char*)h.in[d][k];
             D.out[k] = (char*)h.out[d][k];
             D.x1[k] = (const char*)h.x1[d][k];
@@ -369,7 +378,7 @@ int dd_launch_hop(wl_dd dd, const DDLaunch& h, cudaStream_t s)
         A.max_blocks = dd->part_max_blocks;
     }
     const int extra = (h.x1[0][0] ? 1 : 0) + (h.x2[0][0] ? 1 : 0) + (h.w[0][0] ? 1 : 0);
-    const double site_bytes = (double)(lf ? (P == WL_F32 ? 384 : 192) : link_field_bytes(P, 1)) +
+    const double site_bytes = (double)(lf == 1 ? (P == WL_F32 ? 384 : 192) : link_field_bytes(P, 1)) +
                               (h.cl_mode ? (double)clover_site_bytes(P) : 0.0) + (double)nrhs * (2 + extra) * sb;
     // the interior of a y or z cut as a box (no site list to read)
     bool box_ok = false;

@@ -200,23 +200,6 @@ struct DDArgs {
     DDDom d[kMaxDomains];
 };
 
-// Loop-form spin projection of hop d for the double-float type (the
-// hop_site_loop arithmetic of hop.cuh).
-template <int P, bool DAG>
-__device__ __forceinline__ void project_loop(cx<typename Prec<P>::real> (&h0)[3], cx<typename Prec<P>::real> (&h1)[3],
-                                             const cx<typename Prec<P>::real> (&q)[12], int d)
-{
-    const unsigned code = hop_code(d >> 1);
-    const int sflip = ((d & 1) ? DAG == false : DAG == true) ? 0 : 2;
-    const int a0 = code & 1, k0 = ((code >> 1) + sflip) & 3;
-    const int a1 = (code >> 3) & 1, k1 = ((code >> 4) + sflip) & 3;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        h0[c] = q[c] + mul_ik(a0 ? q[9 + c] : q[6 + c], k0);
-        h1[c] = q[3 + c] + mul_ik(a1 ? q[9 + c] : q[6 + c], k1);
-    }
-}
-
 // One hop of an unrolled site sum: the half spinor from the halo (remote)
 // or projected from the local neighbour.
 template <int P, int D, int MU, int S, int LF, bool HALO>
@@ -236,6 +219,36 @@ __device__ __forceinline__ void dd_hop_one(cx<typename Prec<P>::real> (&acc)[12]
     }
 }
 
+// Hop data of a block site for fixed-point FP64 links: the packed half spinor
+// and the local projection are the same FP64 numbers, so the sums are the
+// undivided kernel's.
+template <bool HALO>
+struct DDFxSrc : FxDirect {
+    const DDArgs& A;
+    unsigned remote;
+    const char* const (&halo)[4][2];
+    const long long (&f)[4];
+
+    __device__ __forceinline__ void half(int k, int mu, double sg, cx<double> (&h0)[3], cx<double> (&h1)[3])
+    {
+        const int hop = fx_order(k);
+        if (HALO && ((remote >> hop) & 1)) {  // (x is never cut: mu > 0)
+            const char* h = hop & 1 ? (mu == 1 ? halo[1][1] : mu == 2 ? halo[2][1] : halo[3][1])
+                                    : (mu == 1 ? halo[1][0] : mu == 2 ? halo[2][0] : halo[3][0]);
+            float unused;
+            load_half<WL_F64>(h0, h1, unused, h, mu == 1 ? A.fs[1] : mu == 2 ? A.fs[2] : A.fs[3],
+                              mu == 1 ? f[1] : mu == 2 ? f[2] : f[3]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                h0[c] = sg * h0[c];
+                h1[c] = sg * h1[c];
+            }
+        } else {
+            FxDirect::half(k, mu, sg, h0, h1);
+        }
+    }
+};
+
 // acc = H in at block site i: like hop_site, with the hops in `remote` read
 // from the halo (halo(mu, side) at face index f[mu]).
 template <int P, bool DAG, int LF, bool HALO>
@@ -245,6 +258,22 @@ __device__ __forceinline__ void dd_hop_site(cx<typename Prec<P>::real> (&acc)[12
 {
     using T = typename Prec<P>::real;
     const long long Vh = A.g.Vh;
+    if constexpr (LF == 3) {
+        FxSum<3> Q;
+        DDFxSrc<HALO> src{{in, Vh, nb, links, Vh, i, 0}, A, remote, halo, f};
+        fx_sum<DAG>(Q, src);
+        const char* hl[6] = {halo[1][0], halo[1][1], halo[2][0], halo[2][1], halo[3][0], halo[3][1]};
+        const long long fs[3] = {A.fs[1], A.fs[2], A.fs[3]}, fi[3] = {f[1], f[2], f[3]};
+        fx_finish<DAG>(acc, Q, links, Vh, i, 0, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
+            if (HALO && ((remote >> d) & 1)) {  // (never the x hops d = 0, 1)
+                float unused;
+                load_half<WL_F64>(h0, h1, unused, hl[d - 2], fs[(d >> 1) - 1], fi[(d >> 1) - 1]);
+            } else {
+                fx_general_local<DAG>(d, h0, h1, in, Vh, fx_pick(nb, d));
+            }
+        });
+        return;
+    }
 #pragma unroll
     for (int c = 0; c < 12; ++c) acc[c] = {(T)0, (T)0};
     if constexpr (P == WL_DF64 && LF == 0) {
@@ -257,7 +286,7 @@ __device__ __forceinline__ void dd_hop_site(cx<typename Prec<P>::real> (&acc)[12
             } else {
                 cx<T> q[12];
                 load_spinor_ro<P>(q, in, Vh, nb[d]);
-                project_loop<P, DAG>(h0, h1, q, d);
+                project_code<T, DAG>(h0, h1, q, d);
             }
             const unsigned code = hop_code(d >> 1);
             const int sflip = ((d & 1) ? DAG == false : DAG == true) ? 0 : 2;
@@ -274,7 +303,7 @@ __device__ __forceinline__ void dd_hop_site(cx<typename Prec<P>::real> (&acc)[12
                 acc[9 + a] = acc[9 + a] + mul_ik(b3 ? u1 : u0, k3);
             }
         }
-    } else {
+    } else if constexpr (LF != 3) {
         constexpr int F = DAG ? +1 : -1;
         constexpr int B = -F;
         const cx<float>* ph = A.ph;

@@ -71,7 +71,7 @@ __device__ __forceinline__ void dd_site(const DDArgs& A, const DDDom& D, int rhs
 // Launches with a fused reduction: a capped grid loops over the sites of both
 // parities, so the per-block partials the finishing launch adds up are few.
 template <int P, bool DAG, bool DOT, int LF, bool BND, int CL>
-__global__ void __launch_bounds__(kDDBlock, (MinBlocks<P, DOT>::value * 2)) dd_hop_kernel(const DDArgs A)
+__global__ void __launch_bounds__(kDDBlock, (MinBlocks<P, DOT, LF>::value * 2)) dd_hop_kernel(const DDArgs A)
 {
     using T = typename Prec<P>::real;
     const int rhs = blockIdx.y, dom = blockIdx.z;
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kDDBlock) dd_pack_kernel(const DDPackArgs A)
     if constexpr (P == WL_DF64) {
         cx<T> q[12];
         load_spinor_ro<P>(q, in, A.g.Vh, i);
-        project_loop<P, DAG>(h0, h1, q, d);
+        project_code<T, DAG>(h0, h1, q, d);
     } else {
         constexpr int F = DAG ? +1 : -1;  // forward projector sign
         constexpr int B = -F;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kDDBlock) dd_pack_kernel(const DDPackArgs A)
 }
 
 // Launchers of one link format and clover mode (LF = 1 exists for FP32 /
-// FP16 only).
+// FP16 only, LF = 3 for FP64).
 template <int LF, int CL>
 struct DDKernels {
     static void hop(int prec, bool dagger, bool dot, bool bnd, const DDArgs& A, dim3 grid, cudaStream_t s);
@@ -196,7 +196,8 @@ static void dd_hop_pb(bool dagger, bool dot, bool bnd, const DDArgs& A, dim3 gri
 template <int LF, int CL>
 void DDKernels<LF, CL>::hop(int prec, bool dagger, bool dot, bool bnd, const DDArgs& A, dim3 grid, cudaStream_t s)
 {
-    if (prec == WL_F32) dd_hop_pb<LF, CL, WL_F32>(dagger, dot, bnd, A, grid, s);
+    if constexpr (LF == 3) dd_hop_pb<LF, CL, WL_F64>(dagger, dot, bnd, A, grid, s);
+    else if (prec == WL_F32) dd_hop_pb<LF, CL, WL_F32>(dagger, dot, bnd, A, grid, s);
     else if (prec == WL_F16) dd_hop_pb<LF, CL, WL_F16>(dagger, dot, bnd, A, grid, s);
     else if constexpr (LF == 0) {
         if (prec == WL_F64) dd_hop_pb<LF, CL, WL_F64>(dagger, dot, bnd, A, grid, s);

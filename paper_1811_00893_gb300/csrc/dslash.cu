@@ -23,12 +23,21 @@ extern template struct HopKernels<kClNone, 1>;
 extern template struct HopKernels<kClX2, 1>;
 extern template struct HopKernels<kClOut, 1>;
 extern template struct HopKernels<kClNone, 2>;  // dslash_r8.cu
+extern template struct HopKernels<kClNone, 3>;  // dslash_fx.cu
+extern template struct HopKernels<kClX2, 3>;    // dslash_fx_clover.cu
+extern template struct HopKernels<kClOut, 3>;
 
 // The kernel family of a launch: clover mode and link format.
 template <typename F>
 static void with_variant(const HopLaunch& h, int lf, F&& f)
 {
-    if (lf == 2) {  // eight-real links: Wilson launches only
+    if (lf == 3) {  // fixed-point FP64 links
+        switch (h.cl_mode) {
+            case kClX2: f(HopKernels<kClX2, 3>()); break;
+            case kClOut: f(HopKernels<kClOut, 3>()); break;
+            default: f(HopKernels<kClNone, 3>()); break;
+        }
+    } else if (lf == 2) {  // eight-real links: Wilson launches only
         f(HopKernels<kClNone, 2>());
     } else if (lf) {
         switch (h.cl_mode) {
@@ -49,7 +58,7 @@ static void with_variant(const HopLaunch& h, int lf, F&& f)
 static size_t link_site_bytes(int prec, int lf)
 {
     if (lf == 2) return 256;
-    if (lf) return prec == WL_F32 ? 384 : 192;
+    if (lf == 1) return prec == WL_F32 ? 384 : 192;
     return link_field_bytes(prec, 1);
 }
 
@@ -100,7 +109,7 @@ static const int kPerRhs = 3000;
 
 static bool rows_allowed(const HopLaunch& h, int lf)
 {
-    return h.prec == WL_F64 && h.cl_mode == kClNone && lf == 0;
+    return h.prec == WL_F64 && h.cl_mode == kClNone && (lf == 0 || lf == 3);
 }
 
 // Resident-block grid of the reducing single-RHS hop kernel.
@@ -126,7 +135,7 @@ static int launch_shape(const HopLaunch& h, int lf, HopArgs& A, int nrhs, int sh
         A.blocks_per_parity = (int)((A.g.Vh + kRowSites - 1) / kRowSites);
         A.partials_only = h.dot ? 1 : 0;
         gx = (unsigned)((long long)A.blocks_per_parity * h.nparity);
-        HopKernels<kClNone, 0>::rows(h.dagger != 0, h.dot, A, dim3(gx, 1), s);
+        with_variant(h, lf, [&](auto K) { K.rows(h.dagger != 0, h.dot, A, dim3(gx, 1), s); });
         if (h.dot)
             return launch_finish_slots(A.red.partial, (long long)A.red.max_blocks * 3, (int)gx, 1, A.dot_out,
                                        A.dot_stride, A.active, A.active_stride, s);
@@ -134,17 +143,17 @@ static int launch_shape(const HopLaunch& h, int lf, HopArgs& A, int nrhs, int sh
         // shapes above kFullGrid: the reducing kernel over the full grid, one
         // site per thread, with a finishing launch for the partial sums
         const bool full = shape > kFullGrid;
-        const int block = full ? shape - kFullGrid : shape;
+        const int block = lf == 3 ? kFxBlock : full ? shape - kFullGrid : shape;
         A.partials_only = h.dot && full ? 1 : 0;
         A.blocks_per_parity = (int)((A.g.Vh + block - 1) / block);
         gx = (unsigned)((long long)A.blocks_per_parity * h.nparity);
-        if (h.dot && !full) gx = std::min(gx, (unsigned)single_grid_cap(h, lf, block));
+        if (h.dot && !full && lf != 3) gx = std::min(gx, (unsigned)single_grid_cap(h, lf, block));
         launch_single(h, lf, A, dim3(gx, 1), block, s);
         if (A.partials_only)
             return launch_finish_slots(A.red.partial, (long long)A.red.max_blocks * 3, (int)gx, 1,
                                        A.dot_out, A.dot_stride, A.active, A.active_stride, s);
-    } else if (shape > kPerRhs) {
-        const int block = shape - kPerRhs;
+    } else if (shape > kPerRhs || lf == 3) {
+        const int block = lf == 3 ? kFxBlock : shape - kPerRhs;
         A.blocks_per_parity = (int)((A.g.Vh + block - 1) / block);
         gx = (unsigned)((long long)A.blocks_per_parity * h.nparity);
         A.partials_only = h.dot ? 1 : 0;
@@ -220,9 +229,14 @@ static int tuned_shape(wl_gauge g, const HopLaunch& h, int lf, HopArgs& A, int n
             return WL_OK;
         }
     }
+    if (multi && lf == 3) return WL_OK;  // one form
     if (!autotune_enabled() || is_capturing(s)) return WL_OK;
     std::vector<int> cand;
-    if (multi) {
+    if (lf == 3) {  // (one site per thread in kFxBlock-thread blocks, or kRowsShape)
+        cand = {kFxBlock};
+        if (h.dot) cand.push_back(kFullGrid + kFxBlock);
+        if (rows_allowed(h, lf)) cand.push_back(kRowsShape);
+    } else if (multi) {
         for (int l : {1, 2, 4, 8})
             if (l <= nrhs) cand.push_back(l);
         if (h.prec == WL_F32 || h.prec == WL_F16) {
@@ -320,12 +334,13 @@ int launch_hop(wl_gauge g, const HopLaunch& h, cudaStream_t s)
     int lf = (h.prec == WL_F32 || h.prec == WL_F16) && g->links_r12[h.prec][0] && !r12_off ? 1 : 0;
     // eight-real links: FP32 single-RHS Wilson launches
     if (h.prec == WL_F32 && g->links_r8[WL_F32][0] && h.nrhs == 1 && h.cl_mode == kClNone && !r12_off) lf = 2;
+    if (h.prec == WL_F64 && g->fx64) lf = 3;
     HopArgs A;
     A.g = g->geo;
     A.partials_only = 0;
     for (int k = 0; k < 2; ++k) {
         const int p = h.parity0 + (k < h.nparity ? k : 0);
-        A.links[k] = lf == 2 ? g->links_r8[h.prec][p] : lf ? g->links_r12[h.prec][p] : g->links[h.prec][p];
+        A.links[k] = lf == 2 ? g->links_r8[h.prec][p] : lf == 1 ? g->links_r12[h.prec][p] : g->links[h.prec][p];
         A.cl[k] = h.clov[k];
     }
     for (int mu = 0; mu < 4; ++mu) A.ph[mu] = {(float)g->bc_re[mu], (float)g->bc_im[mu]};

@@ -1,10 +1,11 @@
 // Gauge objects: validation, the internal link layouts, layout conversion of
 // fermion fields, workspace growth and per-launch timing.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
-#include "internal.cuh"
+#include "hop.cuh"
 
 namespace wl {
 
@@ -112,6 +113,39 @@ __device__ __forceinline__ void store_link<WL_F16>(void* base, long long Vh, int
     q[i] = f2h((float)w[8].re, (float)w[8].im);
 }
 
+// FP64 links as fixed point (LF = 3 of the hopping kernels)
+__device__ void store_link_fx(void* base, long long Vh, int d, long long i, const cx<double> (&w)[9])
+{
+    int4* p = (int4*)base + (long long)d * 9 * Vh;
+    for (int k = 0; k < 9; ++k) {
+        int4 t;
+        fx_split(w[k].re, t.x, t.y);
+        fx_split(w[k].im, t.z, t.w);
+        p[k * Vh + i] = t;
+    }
+}
+
+// The entries of a link are finite and within the modulus that fixed-point
+// storage has room for (a phase factor leaves the modulus alone); in FP32,
+// whose rounding the bound's margin covers many times.
+__device__ bool fx_link_fits(const double* u)
+{
+    bool ok = true;
+    for (int k = 0; k < 9; ++k) {
+        const float re = (float)u[2 * k], im = (float)u[2 * k + 1];
+        ok &= fmaf(re, re, im * im) <= (float)(kFxMaxLink * kFxMaxLink);
+    }
+    return ok;
+}
+
+// The same over all links of a lattice: a block of a decomposition takes the
+// form that the whole lattice's links allow.
+__global__ void __launch_bounds__(256) check_links_kernel(const double* __restrict__ U, long long nlinks, int* flag)
+{
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nlinks; k += (long long)gridDim.x * blockDim.x)
+        if (!fx_link_fits(U + 18 * k)) *flag = 1;
+}
+
 struct BC {
     double re[4], im[4];
 };
@@ -141,8 +175,8 @@ __device__ __forceinline__ long long global_site(const Geom& g, const Place& pl,
     return c[0] + (long long)pl.gl.L[0] * (c[1] + (long long)pl.gl.L[1] * (c[2] + (long long)pl.gl.L[2] * c[3]));
 }
 
-template <int P>
-__global__ void build_links_kernel(void* out, const double* __restrict__ U, Geom g, Place pl, BC bc, int p)
+template <int P, bool FX = false>
+__global__ void build_links_kernel(void* out, const double* __restrict__ U, Geom g, Place pl, BC bc, int p, int* flag = nullptr)
 {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= g.Vh) return;
@@ -155,13 +189,15 @@ __global__ void build_links_kernel(void* out, const double* __restrict__ U, Geom
         cx<double> w[9];
         // forward: phi^[x_mu = L-1] U_mu(x)
         const double* u = U + (s * 4 + mu) * 18;
+        if (FX && !fx_link_fits(u)) *flag = 1;
         double pr = 1.0, pi = 0.0;
         if (c[mu] == G.L[mu] - 1) { pr = bc.re[mu]; pi = bc.im[mu]; }
         for (int k = 0; k < 9; ++k) {
             const double a = u[2 * k], b = u[2 * k + 1];
             w[k] = {pr * a - pi * b, pr * b + pi * a};
         }
-        store_link<P>(out, g.Vh, 2 * mu, i, w);
+        if constexpr (FX) store_link_fx(out, g.Vh, 2 * mu, i, w);
+        else store_link<P>(out, g.Vh, 2 * mu, i, w);
         // backward: conj(phi)^[x_mu = 0] U_mu(x - mu)^dag
         const long long n = (c[mu] == 0) ? s + (G.L[mu] - 1) * stride[mu] : s - stride[mu];
         const double* v = U + (n * 4 + mu) * 18;
@@ -173,7 +209,8 @@ __global__ void build_links_kernel(void* out, const double* __restrict__ U, Geom
                 const double re = v[2 * (b * 3 + a)], im = -v[2 * (b * 3 + a) + 1];
                 w[a * 3 + b] = {pr * re - pi * im, pr * im + pi * re};
             }
-        store_link<P>(out, g.Vh, 2 * mu + 1, i, w);
+        if constexpr (FX) store_link_fx(out, g.Vh, 2 * mu + 1, i, w);
+        else store_link<P>(out, g.Vh, 2 * mu + 1, i, w);
     }
 }
 
@@ -504,12 +541,18 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
         for (int prec = 0; prec < 4 && rc == WL_OK; ++prec) {
             if (!(g->prec_mask & WL_PREC_MASK(prec))) continue;
             for (int p = 0; p < 2; ++p) {
-                cudaError_t e = cudaMalloc(&g->links[prec][p], link_field_bytes(prec, g->geo.Vh));
+                cudaError_t e = cudaMalloc(&g->links[prec][p], link_field_bytes(prec, g->geo.Vh) + 16);
                 if (e != cudaSuccess) {
                     rc = set_error(WL_ERR_CUDA, std::string("cudaMalloc links: ") + cudaGetErrorString(e));
                     break;
                 }
-                if (prec == WL_F64) build_links_kernel<WL_F64><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p);
+                if (prec == WL_F64) {  // fixed point, until a link turns out not to fit (below)
+                    int* flag = (int*)((char*)g->links[prec][p] + link_field_bytes(prec, g->geo.Vh));
+                    cudaMemsetAsync(flag, 0, sizeof(int), s);
+                    build_links_kernel<WL_F64, true><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p, flag);
+                    if (global != local)
+                        check_links_kernel<<<8u * (unsigned)g->num_sms, 256, 0, s>>>(U, 8 * pl.gl.Vh, flag);
+                }
                 else if (prec == WL_F32) build_links_kernel<WL_F32><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p);
                 else if (prec == WL_F16) build_links_kernel<WL_F16><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p);
                 else build_links_kernel<WL_DF64><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p);
@@ -584,6 +627,17 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
                 rc = set_error(WL_ERR_ARG, "WL_LINKS_R8 needs SU(3) links (unitary, det 1, to 1e-6)");
             if (rc != WL_OK) break;
         }
+        int flags[2] = {0, 0};
+        for (int p = 0; p < 2; ++p)
+            cudaMemcpyAsync(&flags[p], (char*)g->links[WL_F64][p] + link_field_bytes(WL_F64, g->geo.Vh), sizeof(int),
+                            cudaMemcpyDeviceToHost, s);
+        if (cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(WL_ERR_CUDA, "link build failed"); break; }
+        g->fx64 = !flags[0] && !flags[1];
+        if (!g->fx64)  // plain FP64 links instead
+            for (int p = 0; p < 2; ++p) {
+                build_links_kernel<WL_F64><<<grid, block, 0, s>>>(g->links[WL_F64][p], U, g->geo, pl, bc, p);
+                count_launch(1, (double)g->geo.Vh * (8 * 144.0 + link_field_bytes(WL_F64, 1)));
+            }
         // the link build reads U: finish before returning so U may be freed
         if (cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(WL_ERR_CUDA, "link build failed"); break; }
     } while (0);

@@ -4,6 +4,8 @@
 // over the eight hops, the fused epilogue and shared-memory link staging.
 #pragma once
 
+#include <type_traits>
+
 #include "clover.cuh"
 #include "internal.cuh"
 
@@ -247,7 +249,8 @@ __device__ __forceinline__ void neighbours(const Geom& g, int p, int i, int (&nb
 // applied to the projected half spinor of boundary-crossing hops.  Twelve
 // reals instead of eighteen per hop: 384 instead of 576 bytes per site in
 // FP32 (192 instead of 288 in FP16).  LF = 2 (FP32, single-RHS launches): eight
-// reals per hop (load_link_r8), 256 bytes per site.
+// reals per hop (load_link_r8), 256 bytes per site.  LF = 3 (FP64): all nine
+// entries as 59-bit fixed point, the size and plane order of LF = 0 (fx64.cuh).
 // ---------------------------------------------------------------------------
 
 template <int P, int LF>
@@ -279,6 +282,10 @@ struct LinkLayout<WL_F16, 1> {  // per hop: 1 uint4 (4 half2) + 1 uint2 (2 half2
 template <>
 struct LinkLayout<WL_F32, 2> {  // per hop: 2 float4 (8 reals)
     static constexpr int n16 = 16, nsmall = 0, small_bytes = 8, bytes = 256;
+};
+template <>
+struct LinkLayout<WL_F64, 3> {  // per entry one int4 (fx64.cuh)
+    static constexpr int n16 = 72, nsmall = 0, small_bytes = 8, bytes = 1152;
 };
 
 // row 2 = conj(row 0 x row 1)
@@ -727,6 +734,36 @@ __device__ __forceinline__ void hop_site_loop(cx<typename Prec<P>::real> (&acc)[
     }
 }
 
+// cp.async (sm_80+): asynchronous copies from global to shared memory
+__device__ __forceinline__ void cp_async16(void* sm, const void* gl)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gl) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* sm, const void* gl)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(a), "l"(gl) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* sm, const void* gl)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(a), "l"(gl) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// wait until at most N committed groups of this thread are still in flight
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+}  // namespace wl
+
+#include "fx64.cuh"
+
+namespace wl {
+
 // acc = H_{p,1-p} in at the output site whose neighbours are nb.  The links
 // are read from planes of stride lVh at index li (the global link field, or a
 // tile of it staged in shared memory).  DAG flips the projector signs.
@@ -741,6 +778,9 @@ __device__ __forceinline__ void hop_site(cx<typename Prec<P>::real> (&acc)[12], 
     using T = typename Prec<P>::real;
     if constexpr (P == WL_DF64 && LF == 0) {
         hop_site_loop<P, DAG>(acc, nb, Vh, in, links, lVh, li);
+    } else if constexpr (LF == 3) {  // (the kernels that have shared memory for it call fx_site_staged)
+        static_assert(P == WL_F64, "fixed-point links are FP64's");
+        fx_site<DAG, 3>(acc, nb, Vh, in, links, lVh, li, 0);
     } else {
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = {(T)0, (T)0};
@@ -841,8 +881,9 @@ __device__ __forceinline__ void epilogue_ptrs(cx<typename Prec<P>::real> (&acc)[
 {
     using T = typename Prec<P>::real;
     const T a = (T)a_;
+    if (P != WL_F64 || a_ != 1.0)  // (FP64: 24 multiplications are a tenth of the hop's pipe time)
 #pragma unroll
-    for (int c = 0; c < 12; ++c) acc[c] = a * acc[c];
+        for (int c = 0; c < 12; ++c) acc[c] = a * acc[c];
     // FP16 operands enter unscaled, their per-site norm folded into one FFMA
     // per value (n = 1 for the other types)
     if (x1) {
@@ -940,29 +981,6 @@ __device__ __forceinline__ void stage_links(char* sm, const char* gl, long long 
 // without waiting; the caller commits them as one group and waits for the
 // group before reading the tile.  Lets a block fetch the next tile's links
 // while it computes on the current one.
-__device__ __forceinline__ void cp_async16(void* sm, const void* gl)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gl) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* sm, const void* gl)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(a), "l"(gl) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* sm, const void* gl)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(a), "l"(gl) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// wait until at most N committed groups of this thread are still in flight
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 template <int P, int LF = 0>
 __device__ __forceinline__ void stage_links_async(char* sm, const char* gl, long long Vh, int base, int n)
 {

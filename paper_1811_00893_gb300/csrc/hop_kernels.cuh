@@ -38,9 +38,10 @@ namespace wl {
 #ifndef WL_MINBLOCKS_DF64
 #define WL_MINBLOCKS_DF64 2
 #endif
-template <int P, bool DOT>
+template <int P, bool DOT, int LF = 0>
 struct MinBlocks {
-    static constexpr int base = P == WL_F64    ? WL_MINBLOCKS_F64
+    static constexpr int base = LF == 3        ? 2  // (the decomposed kernels; hop_fx_kernel has its own)
+                                : P == WL_F64  ? WL_MINBLOCKS_F64
                                 : P == WL_DF64 ? WL_MINBLOCKS_DF64
                                 : P == WL_F32  ? WL_MINBLOCKS_F32
                                                : WL_MINBLOCKS_F16;
@@ -79,7 +80,7 @@ __device__ __forceinline__ void hop_kernel_site(const HopArgs& A, int rhs, int p
     cx<T> acc[12];
     int nb[8];
     unsigned cross = 0;
-    if constexpr (LF >= 1) neighbours(A.g, A.parity0 + pidx, i, nb, cross);
+    if constexpr (LF == 1 || LF == 2) neighbours(A.g, A.parity0 + pidx, i, nb, cross);
     else neighbours(A.g, A.parity0 + pidx, i, nb);
     hop_site<P, DAG, LF>(acc, nb, A.g.Vh, A.in[pidx] + rhs * A.rs_in, A.links[pidx], A.g.Vh, i, cross,
                          A.ph);
@@ -90,7 +91,7 @@ __device__ __forceinline__ void hop_kernel_site(const HopArgs& A, int rhs, int p
 }
 
 template <int P, bool DAG, bool DOT, int CL, int LF>
-__global__ void __launch_bounds__(256, (MinBlocks<P, DOT>::value)) hop_kernel(const HopArgs A)
+__global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_kernel(const HopArgs A)
 {
     const int rhs = blockIdx.y;
     if (A.active && A.active[rhs * A.active_stride] == 0) return;  // uniform per block
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(256, (MinBlocks<P, DOT>::value)) hop_kernel(co
 }
 
 template <int P, bool DAG, bool DOT, int CL, int LF>
-__global__ void __launch_bounds__(256, (MinBlocks<P, DOT>::value)) hop_mrhs_kernel(const HopArgs A, int nrhs)
+__global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_mrhs_kernel(const HopArgs A, int nrhs)
 {
     using T = typename Prec<P>::real;
     extern __shared__ __align__(16) char smem[];
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(256, (MinBlocks<P, DOT>::value)) hop_mrhs_kern
     int nb[8];
     unsigned cross = 0;
     if (valid) {
-        if constexpr (LF >= 1) neighbours(A.g, p, i, nb, cross);
+        if constexpr (LF == 1 || LF == 2) neighbours(A.g, p, i, nb, cross);
         else neighbours(A.g, p, i, nb);
     }
     for (int r = threadIdx.y; r < nrhs; r += blockDim.y) {
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(256, 2) hop_mrhs_pipe_kernel(const HopArgs A, 
         int nb[8];
         unsigned cross = 0;
         if (valid) {
-            if constexpr (LF >= 1) neighbours(A.g, p, i, nb, cross);
+            if constexpr (LF == 1 || LF == 2) neighbours(A.g, p, i, nb, cross);
             else neighbours(A.g, p, i, nb);
         }
         for (int r = threadIdx.y; r < nrhs; r += blockDim.y) {
@@ -262,13 +263,68 @@ __global__ void __launch_bounds__(256, 2) hop_mrhs_pipe_kernel(const HopArgs A, 
     }
 }
 
+// Fixed-point FP64 links (LF = 3): one site per thread, one right-hand side per
+// grid row, the loads of the next hop in flight through cp.async while the
+// present one is computed (FxStaged: 368 bytes of shared memory per thread,
+// which eight resident 64-thread blocks of 128 registers fill to 188 KB).
+// Bound by the issue of integer instructions (~7,300 per warp of sites, 1.9 per
+// clock and SM; DRAM at half its rate), so several right-hand sides gain
+// nothing from sharing the links: a form with the links of a tile staged for
+// all of them took 1,727 us for the hopping term of 24^3 x 48 with 12
+// right-hand sides, one grid row per right-hand side 1,434 us.  32^3 x 64,
+// one right-hand side: 390 us, in FP64 arithmetic 1,628 us.  Reducing
+// launches use the full grid too; the partial sums are added by the last
+// block or (partials_only) by a finishing launch.
+static constexpr int kFxBlock = 64;
+
+template <bool DAG, bool DOT, int CL>
+__global__ void __launch_bounds__(kFxBlock, 8) hop_fx_kernel(const HopArgs A)
+{
+    extern __shared__ __align__(16) char smem[];
+    const int rhs = blockIdx.y;
+    if (A.active && A.active[rhs * A.active_stride] == 0) return;  // uniform per block
+    const int pidx = blockIdx.x / A.blocks_per_parity;
+    const int j = (blockIdx.x - pidx * A.blocks_per_parity) * blockDim.x + threadIdx.x;
+    const bool valid = j < A.g.Vh;
+    const int i = valid ? j : (int)A.g.Vh - 1;  // (whole warps: the staged copies synchronise them)
+    double part[3] = {0, 0, 0};
+    {
+        int nb[8];
+        neighbours(A.g, A.parity0 + pidx, i, nb);
+        cx<double> acc[12];
+        fx_site_staged<DAG>(acc, nb, A.g.Vh, A.in[pidx] + rhs * A.rs_in, (const char*)A.links[pidx], A.g.Vh, i,
+                                  (int4*)smem + (threadIdx.x >> 5) * (FxStaged::kSlots * 32) + (threadIdx.x & 31));
+        if (valid) epilogue<WL_F64, DOT, CL>(acc, A, pidx, rhs, i, part);
+    }
+    if constexpr (DOT) {
+        __shared__ double sh[3 * 32];
+        warp_sum<3>(part);
+        block_sum_warps<3>(part, sh);
+        if (A.partials_only) {
+            if (threadIdx.x == 0)
+                for (int k = 0; k < 3; ++k)
+                    A.red.partial[((long long)rhs * A.red.max_blocks + blockIdx.x) * 3 + k] = part[k];
+            return;
+        }
+        double tot[3];
+        if (grid_sum<3>(part, tot, A.red, rhs, gridDim.x, blockIdx.x, sh)) {
+            double* o = A.dot_out + (long long)rhs * A.dot_stride;
+            o[0] = tot[0];
+            o[1] = tot[1];
+            o[2] = tot[2];
+        }
+    }
+}
+
 // FP64 hopping term for small lattices, where one thread per site leaves
 // most SMs with less than a warp and the kernel's time is the latency of one
 // thread's dependent FP64 chain: three threads per output site, one colour
 // row a each (output components 3 s + a).  Each projects the full neighbour
 // spinors (the three rows read them from L1) and applies row a of every link,
 // a third of hop_kernel's chain per thread and no exchange between the three.
-// Every output component sees hop_kernel's operations in the same order.
+// Every output component sees hop_kernel's operations in the same order (with
+// fixed-point links, hop_fx_kernel's; there one thread per site takes 20 us on
+// 8^4, three threads 14.6 us).
 // Block: kRowSites sites x 3 rows (thread t: row t / kRowSites); a reducing
 // launch leaves one partial per block for the finishing launch.  32 sites per
 // block spread an 8^4 lattice's 2 x 2,048 sites over 128 SMs: on small lattices
@@ -285,7 +341,7 @@ __device__ __forceinline__ void hop_row(cx<double> (&acc)[12], const char* in, l
     reconstruct<MU, S>(acc, 0, dot3(w[0], w[1], w[2], h0), dot3(w[0], w[1], w[2], h1));
 }
 
-template <bool DAG, bool DOT>
+template <bool DAG, bool DOT, int LF>
 __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A)
 {
     const int rhs = blockIdx.y;
@@ -301,18 +357,22 @@ __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A
         const char* in = A.in[pidx] + rhs * A.rs_in;
         const void* links = A.links[pidx];
         cx<double> acc[12];  // the rows of colour a at 0, 3, 6, 9
+        if constexpr (LF == 3) {
+            fx_site<DAG, 1>(acc, nb, Vh, in, links, Vh, i, a);
+        } else {
 #pragma unroll
-        for (int c = 0; c < 12; ++c) acc[c] = {0.0, 0.0};
-        constexpr int F = DAG ? +1 : -1;  // forward projector sign
-        constexpr int B = -F;
-        hop_row<0, 0, F>(acc, in, Vh, nb[0], links, i, a);
-        hop_row<1, 0, B>(acc, in, Vh, nb[1], links, i, a);
-        hop_row<2, 1, F>(acc, in, Vh, nb[2], links, i, a);
-        hop_row<3, 1, B>(acc, in, Vh, nb[3], links, i, a);
-        hop_row<4, 2, F>(acc, in, Vh, nb[4], links, i, a);
-        hop_row<5, 2, B>(acc, in, Vh, nb[5], links, i, a);
-        hop_row<6, 3, F>(acc, in, Vh, nb[6], links, i, a);
-        hop_row<7, 3, B>(acc, in, Vh, nb[7], links, i, a);
+            for (int c = 0; c < 12; ++c) acc[c] = {0.0, 0.0};
+            constexpr int F = DAG ? +1 : -1;  // forward projector sign
+            constexpr int B = -F;
+            hop_row<0, 0, F>(acc, in, Vh, nb[0], links, i, a);
+            hop_row<1, 0, B>(acc, in, Vh, nb[1], links, i, a);
+            hop_row<2, 1, F>(acc, in, Vh, nb[2], links, i, a);
+            hop_row<3, 1, B>(acc, in, Vh, nb[3], links, i, a);
+            hop_row<4, 2, F>(acc, in, Vh, nb[4], links, i, a);
+            hop_row<5, 2, B>(acc, in, Vh, nb[5], links, i, a);
+            hop_row<6, 3, F>(acc, in, Vh, nb[6], links, i, a);
+            hop_row<7, 3, B>(acc, in, Vh, nb[7], links, i, a);
+        }
         // epilogue (as epilogue_ptrs, on this thread's four components)
         auto at = [&](const char* q, long long rs) -> const double2* {
             return q ? (const double2*)(q + rhs * rs) : nullptr;
@@ -324,7 +384,7 @@ __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A
         const double sa = A.a, b1 = A.b1;
         cx<double> v[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) v[s] = sa * acc[3 * s];
+        for (int s = 0; s < 4; ++s) v[s] = sa == 1.0 ? acc[3 * s] : sa * acc[3 * s];
         if (x1)
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
@@ -361,7 +421,8 @@ __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A
 }
 
 // Host-side launchers of one clover mode and link format (LF = 1 exists for
-// FP32 and FP16 only; other precisions are never requested with it).
+// FP32 and FP16 only, LF = 3 for FP64, whose launches all go through single();
+// other precisions are never requested with them).
 template <int CL, int LF = 0>
 struct HopKernels {
     static void single(int prec, bool dagger, bool dot, const HopArgs& A, dim3 grid, int block,
@@ -372,7 +433,7 @@ struct HopKernels {
     static void pipe(int prec, bool dagger, bool dot, const HopArgs& A, int nrhs, int ntiles, dim3 grid,
                      dim3 block, size_t smem, cudaStream_t s);
     static const void* pipe_kernel(int prec, bool dagger, bool dot);
-    // three threads per site (FP64, CL = 0, LF = 0 only), kRowSites sites per block
+    // three threads per site (FP64, CL = 0, LF = 0 or 3), kRowSites sites per block
     static void rows(bool dagger, bool dot, const HopArgs& A, dim3 grid, cudaStream_t s);
     // the reducing single-RHS kernel (for occupancy queries)
     static const void* reducing(int prec, bool dagger);
@@ -400,6 +461,19 @@ static void hop_multi_p(bool dagger, bool dot, const HopArgs& A, int nrhs, dim3 
     } else {
         if (dot) hop_mrhs_kernel<P, false, true, CL, LF><<<grid, block, smem, s>>>(A, nrhs);
         else hop_mrhs_kernel<P, false, false, CL, LF><<<grid, block, smem, s>>>(A, nrhs);
+    }
+}
+
+template <int CL>
+static void hop_fx_single(bool dagger, bool dot, const HopArgs& A, dim3 grid, cudaStream_t s)
+{
+    const size_t smem = FxStaged::kSlots * 16 * kFxBlock;
+    if (dagger) {
+        if (dot) hop_fx_kernel<true, true, CL><<<grid, kFxBlock, smem, s>>>(A);
+        else hop_fx_kernel<true, false, CL><<<grid, kFxBlock, smem, s>>>(A);
+    } else {
+        if (dot) hop_fx_kernel<false, true, CL><<<grid, kFxBlock, smem, s>>>(A);
+        else hop_fx_kernel<false, false, CL><<<grid, kFxBlock, smem, s>>>(A);
     }
 }
 
@@ -451,6 +525,8 @@ void HopKernels<CL, LF>::single(int prec, bool dagger, bool dot, const HopArgs& 
 {
     if constexpr (LF == 2) {
         if (prec == WL_F32) hop_single_p<CL, LF, WL_F32>(dagger, dot, A, grid, block, s);
+    } else if constexpr (LF == 3) {
+        if (prec == WL_F64) hop_fx_single<CL>(dagger, dot, A, grid, s);
     } else {
         if (prec == WL_F32) hop_single_p<CL, LF, WL_F32>(dagger, dot, A, grid, block, s);
         else if (prec == WL_F16) hop_single_p<CL, LF, WL_F16>(dagger, dot, A, grid, block, s);
@@ -478,14 +554,14 @@ void HopKernels<CL, LF>::multi(int prec, bool dagger, bool dot, const HopArgs& A
 template <int CL, int LF>
 void HopKernels<CL, LF>::rows(bool dagger, bool dot, const HopArgs& A, dim3 grid, cudaStream_t s)
 {
-    if constexpr (CL == kClNone && LF == 0) {
+    if constexpr (CL == kClNone && (LF == 0 || LF == 3)) {
         const int block = 3 * kRowSites;
         if (dagger) {
-            if (dot) hop_rows_kernel<true, true><<<grid, block, 0, s>>>(A);
-            else hop_rows_kernel<true, false><<<grid, block, 0, s>>>(A);
+            if (dot) hop_rows_kernel<true, true, LF><<<grid, block, 0, s>>>(A);
+            else hop_rows_kernel<true, false, LF><<<grid, block, 0, s>>>(A);
         } else {
-            if (dot) hop_rows_kernel<false, true><<<grid, block, 0, s>>>(A);
-            else hop_rows_kernel<false, false><<<grid, block, 0, s>>>(A);
+            if (dot) hop_rows_kernel<false, true, LF><<<grid, block, 0, s>>>(A);
+            else hop_rows_kernel<false, false, LF><<<grid, block, 0, s>>>(A);
         }
     }
 }
@@ -493,7 +569,9 @@ void HopKernels<CL, LF>::rows(bool dagger, bool dot, const HopArgs& A, dim3 grid
 template <int CL, int LF>
 const void* HopKernels<CL, LF>::reducing(int prec, bool dagger)
 {
-    if (prec == WL_F32)
+    if constexpr (LF == 3)
+        return nullptr;  // (full grids only)
+    else if (prec == WL_F32)
         return dagger ? (const void*)hop_kernel<WL_F32, true, true, CL, LF> : (const void*)hop_kernel<WL_F32, false, true, CL, LF>;
     if constexpr (LF < 2) {
         if (prec == WL_F16)
