@@ -119,6 +119,24 @@ __global__ void __launch_bounds__(256) cdot_kernel(const void* a, const void* b,
     }
 }
 
+// value conversions between the storage types; FP64 <-> FP32 on the integer
+// pipes (df64.cuh), which are faster than the FP64 pipe's conversions
+template <typename TD, typename TS>
+__device__ __forceinline__ TD cast(TS v)
+{
+    return (TD)v;
+}
+template <>
+__device__ __forceinline__ float cast<float, double>(double v)
+{
+    return narrow_f64(v);
+}
+template <>
+__device__ __forceinline__ double cast<double, float>(float v)
+{
+    return widen_f32(v);
+}
+
 template <int PD, int PS>
 __global__ void convert_kernel(void* dst, Vec vd, const void* src, Vec vs, const int* mask)
 {
@@ -132,7 +150,7 @@ __global__ void convert_kernel(void* dst, Vec vd, const void* src, Vec vs, const
     cx<typename Prec<PD>::real> y[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c)
-        y[c] = {(typename Prec<PD>::real)x[c].re, (typename Prec<PD>::real)x[c].im};
+        y[c] = {cast<typename Prec<PD>::real>(x[c].re), cast<typename Prec<PD>::real>(x[c].im)};
     store_spinor<PD>((void*)at(dst, vd, rhs, j, i), vd.Vh, i, y);
 }
 
@@ -166,7 +184,7 @@ __global__ void accum_hi_kernel(void* xhi, Vec vh, const void* xlo, Vec vl, cons
     char* ph = (char*)at(xhi, vh, rhs, j, i);
     load_spinor<PH>(y, ph, vh.Vh, i);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) y[c] = {y[c].re + (TH)x[c].re, y[c].im + (TH)x[c].im};
+    for (int c = 0; c < 12; ++c) y[c] = {y[c].re + cast<TH>(x[c].re), y[c].im + cast<TH>(x[c].im)};
     store_spinor<PH>(ph, vh.Vh, i, y);
 }
 

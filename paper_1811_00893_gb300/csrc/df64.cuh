@@ -47,6 +47,21 @@ __device__ __forceinline__ double widen_f32(float f)
     return __longlong_as_double((long long)bits);
 }
 
+// binary64 -> binary32, round to nearest even, for zeros and for biased exponents
+// E in [949, 1149] (2^-74 <= |v| < 2^127) from the encoding: the 53-bit
+// significand rounded to 24 bits, a carry running into the exponent field as
+// the format provides; other values take the hardware conversion.
+__device__ __forceinline__ float narrow_f64(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned E = (unsigned)(b >> 52) & 0x7ffu;
+    if (E - 949u > 200u) return __double2float_rn(v);
+    const unsigned low = (unsigned)b & 0x1fffffffu;
+    const unsigned up = (unsigned)(b >> 29) & 0x7fffffu;
+    const unsigned rnd = (low + 0xfffffffu + (up & 1u)) >> 29;  // 1 above half, or at half with an odd last bit kept
+    return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | ((((E - 896u) << 23) | up) + rnd));
+}
+
 struct df64 {
     float hi, lo;
 

@@ -241,7 +241,12 @@ static int ws_alloc(void** p, size_t bytes)
 int ensure_ws(wl_gauge g, int inner, int nrhs, int eo)
 {
     Workspace* w = g->ws;
-    if (w && w->inner == inner && w->nrhs >= nrhs && w->eo == eo) return WL_OK;
+    // Outer residual corrections of mixed-precision solves.  FP64 with
+    // fixed-point links (fx64.cuh): 32^3 x 64 hopping term 390 us, in df64
+    // (double-float) 455 us, and b and x need no second copy.  df64 for links that do not fit, and with a clover term,
+    // whose 6x6 products stay on the FP64 pipe.
+    const int outer = inner == WL_F64 || (g->fx64 && !g->has_clover) ? WL_F64 : WL_DF64;
+    if (w && w->inner == inner && w->nrhs >= nrhs && w->eo == eo && w->outer == outer) return WL_OK;
     WL_CUDA(cudaDeviceSynchronize());
     free_workspace(g);
     g->ws = new Workspace();
@@ -251,9 +256,7 @@ int ensure_ws(wl_gauge g, int inner, int nrhs, int eo)
     w->eo = eo;
     w->nhalf = eo ? 1 : 2;
     w->xlo_prec = inner == WL_F64 ? WL_F64 : WL_F32;
-    // outer residual corrections of mixed-precision solves in df64 (FP32-rate
-    // arithmetic, ~2^-44 rounding); the plain FP64 solve stays in FP64
-    w->outer = inner == WL_F64 ? WL_F64 : WL_DF64;
+    w->outer = outer;
     const long long Vh = g->geo.Vh;
     w->vb = spinor_field_bytes(inner, Vh) * w->nhalf;
     w->hb64 = spinor_field_bytes(WL_F64, Vh);
