@@ -84,29 +84,35 @@ __global__ void __launch_bounds__(256) cdot_kernel(const void* a, const void* b,
     using T = typename Prec<P>::real;
     const int rhs = blockIdx.y;
     if (mask && !mask[rhs]) return;
-    double part[3] = {0, 0, 0};  // per-site FP64 accumulation (off the hot path)
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < v.nhalf * v.Vh;
-         j += (long long)gridDim.x * blockDim.x) {
-        long long i;
-        cx<T> x[12], y[12];
-        load_spinor<P>(y, at(b, v, rhs, j, i), v.Vh, i);
-        T cr = 0, ci = 0, nn = 0;
-        if (NORM) {
+    double part[3] = {0, 0, 0};  // per-site sums added in FP64
+    constexpr int U = NORM && P != WL_F64 && P != WL_DF64 ? 4 : 2;  // sites in flight per thread
+    const long long total = v.nhalf * v.Vh, step = (long long)gridDim.x * blockDim.x;
+    for (long long j0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; j0 < total; j0 += U * step) {
+        cx<T> x[NORM ? 1 : U][12], y[U][12];
 #pragma unroll
-            for (int c = 0; c < 12; ++c) nn = fma(y[c].re, y[c].re, fma(y[c].im, y[c].im, nn));
-            cr = nn;
-        } else {
-            load_spinor<P>(x, at(a, v, rhs, j, i), v.Vh, i);
+        for (int u = 0; u < U; ++u) {
+            const long long j = min(j0 + u * step, total - 1);
+            long long i;
+            load_spinor<P>(y[u], at(b, v, rhs, j, i), v.Vh, i);
+            if constexpr (!NORM) load_spinor<P>(x[u], at(a, v, rhs, j, i), v.Vh, i);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (j0 + u * step >= total) break;
+            T cr = 0, ci = 0, nn = 0;
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
-                cr = fma(x[c].re, y[c].re, fma(x[c].im, y[c].im, cr));
-                ci = fma(x[c].re, y[c].im, fma(-x[c].im, y[c].re, ci));
-                nn = fma(y[c].re, y[c].re, fma(y[c].im, y[c].im, nn));
+                if constexpr (!NORM) {
+                    cr = fma(x[u][c].re, y[u][c].re, fma(x[u][c].im, y[u][c].im, cr));
+                    ci = fma(x[u][c].re, y[u][c].im, fma(-x[u][c].im, y[u][c].re, ci));
+                }
+                nn = fma(y[u][c].re, y[u][c].re, fma(y[u][c].im, y[u][c].im, nn));
             }
+            if constexpr (NORM) cr = nn;
+            part[0] += (double)cr;
+            part[1] += (double)ci;
+            part[2] += (double)nn;
         }
-        part[0] += (double)cr;
-        part[1] += (double)ci;
-        part[2] += (double)nn;
     }
     __shared__ double sh[3 * 32];
     block_sum<3>(part, sh);
@@ -117,24 +123,6 @@ __global__ void __launch_bounds__(256) cdot_kernel(const void* a, const void* b,
         o[1] = tot[1];
         o[2] = tot[2];
     }
-}
-
-// value conversions between the storage types; FP64 <-> FP32 on the integer
-// pipes (df64.cuh), which are faster than the FP64 pipe's conversions
-template <typename TD, typename TS>
-__device__ __forceinline__ TD cast(TS v)
-{
-    return (TD)v;
-}
-template <>
-__device__ __forceinline__ float cast<float, double>(double v)
-{
-    return narrow_f64(v);
-}
-template <>
-__device__ __forceinline__ double cast<double, float>(float v)
-{
-    return widen_f32(v);
 }
 
 template <int PD, int PS>
@@ -214,7 +202,9 @@ int launch_cdot(wl_gauge g, int prec, const void* a, const void* b, int nhalf, i
                        : prec == WL_F32 ? (const void*)cdot_kernel<WL_F32, false>
                        : prec == WL_F16 ? (const void*)cdot_kernel<WL_F16, false>
                                         : (const void*)cdot_kernel<WL_DF64, false>;
-    grid.x = std::min(grid.x, (unsigned)resident_grid(kern, kBlasBlock, 0));
+    // resident blocks in all: the FP64 sums over a block's threads cost more
+    // than a few sites' loads
+    grid.x = std::min(grid.x, (unsigned)((resident_grid(kern, kBlasBlock, 0) + nrhs - 1) / nrhs));
     WL_TRY(ensure_red(g, nrhs, grid.x));
     const Vec v = make_vec(g, prec, nhalf, rs);
     auto go = [&](auto nt) {

@@ -430,6 +430,24 @@ __device__ __forceinline__ void load_link<WL_F16>(cx<float> (&w)[9], const void*
     w[8] = {t.x, t.y};
 }
 
+// value conversions between the storage types; FP64 <-> FP32 on the integer
+// pipes (df64.cuh), which are faster than the FP64 pipe's conversions
+template <typename TD, typename TS>
+__device__ __forceinline__ TD cast(TS v)
+{
+    return (TD)v;
+}
+template <>
+__device__ __forceinline__ float cast<float, double>(double v)
+{
+    return narrow_f64(v);
+}
+template <>
+__device__ __forceinline__ double cast<double, float>(float v)
+{
+    return widen_f32(v);
+}
+
 // ---------------------------------------------------------------------------
 // reductions: warp shuffle -> shared memory -> per-block partial in FP64 ->
 // the last block to finish (atomic ticket) sums the partials in a fixed

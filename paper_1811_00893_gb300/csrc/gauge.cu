@@ -334,35 +334,102 @@ __global__ void build_links_r8_kernel(void* out, const double* __restrict__ U, G
 // fermion layout conversion
 // ---------------------------------------------------------------------------
 
-template <int P>
-__global__ void to_internal_kernel(char* out, const double* __restrict__ in, Geom g, int p,
-                                   size_t fb, long long V)
+// A canonical site is 192 contiguous bytes, every other site of a row belongs
+// to the other parity, and an internal field has one plane per component (pair):
+// one thread per site on the canonical side would touch 32 sites' 192-byte
+// runs with each warp access.  A block moves kConvSites sites through shared
+// memory instead: 12 consecutive threads move one site's 12 complex numbers on the
+// canonical side, one thread per site its planes on the internal side.  HBM
+// bound, on runs of 192 bytes every 384: FP32, 24^3 x 48, 12 right-hand sides
+// (1.15 GB either way, 169 us at the copy rate): to canonical 666 us with one
+// thread per site, 212 us so; to
+// internal 264 us, 259 us (288 us without cp.async).  The FP64 <-> FP32 conversions run on the integer pipes (df64.cuh).
+static constexpr int kConvSites = 128;
+static constexpr int kConvPitch = kConvSites + 1;  // 16-byte words: neighbouring components in different banks
+
+// canonical index of half site i of parity p, by the fast divisions (below 2^31)
+__device__ __forceinline__ long long canonical_site(const Geom& g, int p, int i)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int rhs = blockIdx.y;
-    if (i >= g.Vh) return;
-    const long long s = site_of_half(g, p, i);
-    const double* q = in + ((long long)rhs * V + s) * 24;
-    cx<typename Prec<P>::real> v[12];
-    for (int c = 0; c < 12; ++c)
-        v[c] = {(typename Prec<P>::real)q[2 * c], (typename Prec<P>::real)q[2 * c + 1]};
-    store_spinor<P>(out + rhs * fb, g.Vh, i, v);
+    const int r0 = geo_div(g, 0, i);
+    const int r1 = geo_div(g, 1, r0);
+    const int y = r0 - r1 * g.L[1];
+    const int t = geo_div(g, 2, r1);
+    const int z = r1 - t * g.L[2];
+    return 2 * (long long)i + ((p + y + z + t) & 1);
 }
 
 template <int P>
-__global__ void to_canonical_kernel(double* out, const char* in, Geom g, int p, size_t fb,
-                                    long long V)
+__global__ void __launch_bounds__(kConvSites) to_internal_kernel(char* out, const double* __restrict__ in, Geom g, int p,
+                                                                 size_t fb, long long V)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const int rhs = blockIdx.y;
-    if (i >= g.Vh) return;
-    const long long s = site_of_half(g, p, i);
-    double* q = out + ((long long)rhs * V + s) * 24;
-    cx<typename Prec<P>::real> v[12];
-    load_spinor<P>(v, in + rhs * fb, g.Vh, i);
+    __shared__ double2 sm[12 * kConvPitch];
+    __shared__ unsigned where[kConvSites];
+    const int rhs = blockIdx.y, base = blockIdx.x * kConvSites;
+    const int n = (int)min((long long)kConvSites, g.Vh - base);
+    if ((int)threadIdx.x < n) where[threadIdx.x] = (unsigned)canonical_site(g, p, base + threadIdx.x);
+    __syncthreads();
+    if (((size_t)in & 15) == 0) {  // cp.async: every copy of the block in flight, no register waits
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const int e = k * kConvSites + threadIdx.x, j = e / 12, c = e - 12 * j;
+            if (j < n) cp_async16(sm + c * kConvPitch + j, in + (((long long)rhs * V + where[j]) * 12 + c) * 2);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+    } else {  // callers' fields are aligned to 8 bytes at least
+        for (int k = 0; k < 12; ++k) {
+            const int e = k * kConvSites + threadIdx.x, j = e / 12, c = e - 12 * j;
+            if (j >= n) break;
+            const double* q = in + (((long long)rhs * V + where[j]) * 12 + c) * 2;
+            sm[c * kConvPitch + j] = make_double2(__ldg(q), __ldg(q + 1));
+        }
+    }
+    __syncthreads();
+    if ((int)threadIdx.x >= n) return;
+    using T = typename Prec<P>::real;
+    cx<T> v[12];
+#pragma unroll
     for (int c = 0; c < 12; ++c) {
-        q[2 * c] = (double)v[c].re;
-        q[2 * c + 1] = (double)v[c].im;
+        const double2 u = sm[c * kConvPitch + threadIdx.x];
+        v[c] = {cast<T>(u.x), cast<T>(u.y)};
+    }
+    store_spinor<P>(out + rhs * fb, g.Vh, base + threadIdx.x, v);
+}
+
+// (the narrow types pass through shared memory in FP32: half the space, twice the resident blocks)
+template <int P>
+__global__ void __launch_bounds__(kConvSites) to_canonical_kernel(double* out, const char* in, Geom g, int p, size_t fb,
+                                                                  long long V)
+{
+    constexpr bool narrow = P == WL_F32 || P == WL_F16;
+    using W = typename std::conditional<narrow, float2, double2>::type;
+    using S = typename std::conditional<narrow, float, double>::type;
+    __shared__ W sm[12 * kConvPitch];
+    __shared__ unsigned where[kConvSites];
+    const int rhs = blockIdx.y, base = blockIdx.x * kConvSites;
+    const int n = (int)min((long long)kConvSites, g.Vh - base);
+    if ((int)threadIdx.x < n) {
+        cx<typename Prec<P>::real> v[12];
+        load_spinor<P>(v, in + rhs * fb, g.Vh, base + threadIdx.x);
+        where[threadIdx.x] = (unsigned)canonical_site(g, p, base + threadIdx.x);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) sm[c * kConvPitch + threadIdx.x] = {cast<S>(v[c].re), cast<S>(v[c].im)};
+    }
+    __syncthreads();
+    const bool wide = ((size_t)out & 15) == 0;  // callers' fields are aligned to 8 bytes at least
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const int e = k * kConvSites + threadIdx.x, j = e / 12, c = e - 12 * j;
+        if (j >= n) continue;
+        double* q = out + (((long long)rhs * V + where[j]) * 12 + c) * 2;
+        const W u = sm[c * kConvPitch + j];
+        const double2 d = make_double2(cast<double>(u.x), cast<double>(u.y));
+        if (wide) {
+            *(double2*)q = d;
+        } else {
+            q[0] = d.x;
+            q[1] = d.y;
+        }
     }
 }
 
@@ -731,7 +798,7 @@ namespace wl {
 int field_to_internal(wl_gauge g, void* out, const double* in, int parity, int prec, int nrhs,
                       cudaStream_t s, long long out_rs)
 {
-    const int block = 128;
+    const int block = kConvSites;
     dim3 grid((unsigned)((g->geo.Vh + block - 1) / block), (unsigned)nrhs);
     const size_t fb = out_rs > 0 ? (size_t)out_rs : spinor_field_bytes(prec, g->geo.Vh);
     const long long V = 2 * g->geo.Vh;
@@ -748,7 +815,7 @@ int field_to_internal(wl_gauge g, void* out, const double* in, int parity, int p
 int field_to_canonical(wl_gauge g, double* out, const void* in, int parity, int prec, int nrhs,
                        cudaStream_t s, long long in_rs)
 {
-    const int block = 128;
+    const int block = kConvSites;
     dim3 grid((unsigned)((g->geo.Vh + block - 1) / block), (unsigned)nrhs);
     const size_t fb = in_rs > 0 ? (size_t)in_rs : spinor_field_bytes(prec, g->geo.Vh);
     const long long V = 2 * g->geo.Vh;
