@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(256) batch_update_p_kernel(const BatchArgs B)
     if (i >= L.g.Vh) return;
     const long long o = ls.y * L.vb;
     const double c[4] = {coef[0], coef[1], coef[2], coef[3]};
-    p_update_site<P>(L.p + o, L.r + o, L.v + o, L.g.Vh, i, c);
+    p_update_site<P>(L.p + o, L.r + o, L.v + o, L.g.Vh, i, c, S.fresh != 0);
 }
 
 template <int P>
@@ -262,13 +262,14 @@ __global__ void __launch_bounds__(256) batch_update_xr_kernel(const BatchArgs B)
     }
     __syncthreads();
     const double dc[4] = {dcoef[0], dcoef[1], dcoef[2], dcoef[3]};
+    const bool fresh = S.fresh != 0;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     using T = typename Prec<P>::real;
     T pt[3] = {0, 0, 0};
     if (i < L.g.Vh) {
         const long long o = ls.y * L.vb;
         xr_update_site<P, PX>(L.xlo + ls.y * L.xb, L.r + o, L.p + o, L.s + o, L.t + o, L.rh + o,
-                              L.g.Vh, i, dc, pt);
+                              L.g.Vh, i, dc, pt, fresh);
     }
     // warp totals in the arithmetic type (FP32 for the narrow types), FP64 from there
     typename RedType<T>::type wp[3] = {(typename RedType<T>::type)pt[0], (typename RedType<T>::type)pt[1],

@@ -156,23 +156,34 @@ __global__ void zero_kernel(void* dst, Vec v, const int* mask)
     store_spinor<P>((void*)at(dst, v, rhs, j, i), v.Vh, i, y);
 }
 
-// x_hi (FP64 or df64) += x_lo
+// x_hi (FP64 or df64) += x_lo; set: x_hi = x_lo for the masked right-hand sides, 0 for the others
 template <int PH, int PL>
-__global__ void accum_hi_kernel(void* xhi, Vec vh, const void* xlo, Vec vl, const int* mask)
+__global__ void accum_hi_kernel(void* xhi, Vec vh, const void* xlo, Vec vl, const int* mask, bool set)
 {
     using TH = typename Prec<PH>::real;
     const int rhs = blockIdx.y;
-    if (mask && !mask[rhs]) return;
+    const bool add = !mask || mask[rhs];
+    if (!add && !set) return;
     const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (j >= vh.nhalf * vh.Vh) return;
     long long i;
-    cx<typename Prec<PL>::real> x[12];
-    load_spinor<PL>(x, at(xlo, vl, rhs, j, i), vl.Vh, i);
     cx<TH> y[12];
     char* ph = (char*)at(xhi, vh, rhs, j, i);
-    load_spinor<PH>(y, ph, vh.Vh, i);
+    if (set) {
 #pragma unroll
-    for (int c = 0; c < 12; ++c) y[c] = {y[c].re + cast<TH>(x[c].re), y[c].im + cast<TH>(x[c].im)};
+        for (int c = 0; c < 12; ++c) y[c] = {TH(0), TH(0)};
+    } else {
+        load_spinor<PH>(y, ph, vh.Vh, i);
+    }
+    if (add) {
+        cx<typename Prec<PL>::real> x[12];
+        load_spinor<PL>(x, at(xlo, vl, rhs, j, i), vl.Vh, i);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            if (set) y[c] = {cast<TH>(x[c].re), cast<TH>(x[c].im)};
+            else y[c] = {y[c].re + cast<TH>(x[c].re), y[c].im + cast<TH>(x[c].im)};
+        }
+    }
     store_spinor<PH>(ph, vh.Vh, i, y);
 }
 
@@ -258,20 +269,20 @@ int launch_zero(wl_gauge g, int prec, void* dst, int nhalf, int nrhs, const int*
 
 template <int PH>
 static void accum_from(int plo, void* xhi, Vec vh, const void* xlo, Vec vl, dim3 grid,
-                       const int* mask, cudaStream_t s)
+                       const int* mask, cudaStream_t s, bool set)
 {
-    if (plo == WL_F64) accum_hi_kernel<PH, WL_F64><<<grid, kBlasBlock, 0, s>>>(xhi, vh, xlo, vl, mask);
-    else if (plo == WL_F32) accum_hi_kernel<PH, WL_F32><<<grid, kBlasBlock, 0, s>>>(xhi, vh, xlo, vl, mask);
-    else accum_hi_kernel<PH, WL_F16><<<grid, kBlasBlock, 0, s>>>(xhi, vh, xlo, vl, mask);
+    if (plo == WL_F64) accum_hi_kernel<PH, WL_F64><<<grid, kBlasBlock, 0, s>>>(xhi, vh, xlo, vl, mask, set);
+    else if (plo == WL_F32) accum_hi_kernel<PH, WL_F32><<<grid, kBlasBlock, 0, s>>>(xhi, vh, xlo, vl, mask, set);
+    else accum_hi_kernel<PH, WL_F16><<<grid, kBlasBlock, 0, s>>>(xhi, vh, xlo, vl, mask, set);
 }
 
 int launch_accum_hi(wl_gauge g, int phi, void* xhi, int plo, const void* xlo, int nhalf, int nrhs,
-                    const int* mask, cudaStream_t s, long long hi_rs)
+                    const int* mask, cudaStream_t s, long long hi_rs, bool set)
 {
     const dim3 grid = blas_grid(g, nhalf, nrhs);
     const Vec vh = make_vec(g, phi, nhalf, hi_rs), vl = make_vec(g, plo, nhalf);
-    if (phi == WL_DF64) accum_from<WL_DF64>(plo, xhi, vh, xlo, vl, grid, mask, s);
-    else accum_from<WL_F64>(plo, xhi, vh, xlo, vl, grid, mask, s);
+    if (phi == WL_DF64) accum_from<WL_DF64>(plo, xhi, vh, xlo, vl, grid, mask, s, set);
+    else accum_from<WL_F64>(plo, xhi, vh, xlo, vl, grid, mask, s, set);
     WL_CHECK_LAUNCH((double)(2 * vh.hb + vl.hb) * nhalf * nrhs);
     return WL_OK;
 }

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kDDVec) dd_update_p_kernel(const DDVecs V)
     if (i >= V.Vh) return;
     const long long o = rhs * V.rs;
     const double c[4] = {coef[0], coef[1], coef[2], coef[3]};
-    p_update_site<P>(V.a[dom] + o, V.b[dom] + o, V.c[dom] + o, V.Vh, i, c);
+    p_update_site<P>(V.a[dom] + o, V.b[dom] + o, V.c[dom] + o, V.Vh, i, c, false);
 }
 
 // s = r - alpha v:  a = s, b = r, c = v
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kDDVec) dd_update_xr_kernel(const DDVecs V)
     for (long long i = blockIdx.x * (long long)kDDVec + threadIdx.x; i < V.Vh; i += (long long)gridDim.x * kDDVec) {
         T q[3];
         xr_update_site<P, PX>(V.x[dom] + rhs * V.rsx, V.a[dom] + o, V.b[dom] + o, V.c[dom] + o, V.d[dom] + o,
-                              V.e[dom] + o, V.Vh, i, dc, q);
+                              V.e[dom] + o, V.Vh, i, dc, q, false);
         for (int k = 0; k < 3; ++k) pt[k] += q[k];
     }
     typename RedType<T>::type wp[3] = {(typename RedType<T>::type)pt[0], (typename RedType<T>::type)pt[1],

@@ -170,8 +170,9 @@ int launch_convert(wl_gauge g, int pdst, void* dst, int psrc, const void* src, i
 int launch_zero(wl_gauge g, int prec, void* dst, int nhalf, int nrhs, const int* mask,
                 cudaStream_t s);
 // x_hi (precision phi: FP64 or df64) += x_lo (precision plo)
+// (set: x_hi = x_lo for the masked right-hand sides, 0 for the others)
 int launch_accum_hi(wl_gauge g, int phi, void* xhi, int plo, const void* xlo, int nhalf, int nrhs,
-                    const int* mask, cudaStream_t s, long long hi_rs = 0);
+                    const int* mask, cudaStream_t s, long long hi_rs = 0, bool set = false);
 
 bool is_capturing(cudaStream_t s);
 

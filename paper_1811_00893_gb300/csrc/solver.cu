@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256) update_p_kernel(char* p, const char* r, c
     const long long i = split_index(vec, j, off);
     off += rhs * vec.rstride;
     const double c[4] = {coef[0], coef[1], coef[2], coef[3]};
-    p_update_site<P>(p + off, r + off, v + off, vec.Vh, i, c);
+    p_update_site<P>(p + off, r + off, v + off, vec.Vh, i, c, S.fresh != 0);
 }
 
 template <int P>
@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(256) update_xr_kernel(char* x, Vec2 vx, char* 
     __syncthreads();
     using T = typename Prec<P>::real;
     const double dc[4] = {dcoef[0], dcoef[1], dcoef[2], dcoef[3]};
+    const bool fresh = S.fresh != 0;
     T tpart[3] = {0, 0, 0};  // this thread's sites in the kernel's arithmetic
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < vec.nhalf * vec.Vh;
          j += (long long)gridDim.x * blockDim.x) {
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(256) update_xr_kernel(char* x, Vec2 vx, char* 
         offx += rhs * vx.rstride;
         T pt[3];
         xr_update_site<P, PX>(x + offx, r + off, p + off, s + off, t + off, rh + off, vec.Vh, i,
-                              dc, pt);
+                              dc, pt, fresh);
         for (int k = 0; k < 3; ++k) tpart[k] += pt[k];
     }
     typename RedType<T>::type wp[3] = {(typename RedType<T>::type)tpart[0],
@@ -185,26 +186,68 @@ __global__ void __launch_bounds__(256) update_xr_kernel(char* x, Vec2 vx, char* 
     if (grid_sum<3>(part, tot, red, rhs, gridDim.x, blockIdx.x, sh)) advance_scalars(S, tot, dc);
 }
 
-// Start (or restart) the scalars of the masked right-hand sides; rr holds
-// (rhat, r) and ||r||^2 from a preceding cdot.
-__global__ void init_scal_kernel(Scal* sc, const int* mask, int nrhs, int full)
+// Scalars after the residual was replaced: rr holds (rhat, r) and ||r||^2
+__device__ __forceinline__ void restart_scalars(Scal& S)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nrhs || !mask[k]) return;
-    Scal& S = sc[k];
-    if (full) {
-        S.rho_prev[0] = 1.0;
-        S.rho_prev[1] = 0.0;
-        S.alpha[0] = 1.0;
-        S.alpha[1] = 0.0;
-        S.omega[0] = 1.0;
-        S.omega[1] = 0.0;
-        S.rh2 = S.rr[2];
-    }
     S.r2_max = S.rr[2];
     S.want_update = 0;
     S.active = S.rr[2] > S.target2 ? 1 : 0;
     if (!S.active) S.flags |= FLAG_CONVERGED;
+}
+
+// The same for the masked right-hand sides after a reliable update (rr from a
+// preceding cdot)
+__global__ void restart_scal_kernel(Scal* sc, const int* mask, int nrhs)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nrhs || !mask[k]) return;
+    restart_scalars(sc[k]);
+}
+
+// Start a round for the masked right-hand sides: r = rhat = the outer residual
+// (precision PS) rounded to P, ||r||^2 of the rounded r and fresh scalars, in one
+// pass: p, v and x_lo need no zeroing (Scal::fresh).  Separate conversion, copy,
+// three fills and a dot product moved 960 bytes per FP32 site from an FP64
+// residual, this 384.
+template <int P, int PS>
+__global__ void __launch_bounds__(256) round_start_kernel(char* r, char* rh, Vec2 v, const char* src, Vec2 vs,
+                                                          const int* mask, Scal* sc, RedScratch red)
+{
+    const int rhs = blockIdx.y;
+    if (!mask[rhs]) return;
+    using T = typename Prec<P>::real;
+    double part[1] = {0.0};
+    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < v.nhalf * v.Vh;
+         j += (long long)gridDim.x * blockDim.x) {
+        long long off, offs;
+        const long long i = split_index(v, j, off);
+        split_index(vs, j, offs);
+        off += rhs * v.rstride;
+        cx<typename Prec<PS>::real> x[12];
+        load_spinor<PS>(x, src + offs + rhs * vs.rstride, v.Vh, i);
+        cx<T> y[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) y[c] = {cast<T>(x[c].re), cast<T>(x[c].im)};
+        store_spinor<P>(r + off, v.Vh, i, y);
+        store_spinor<P>(rh + off, v.Vh, i, y);
+        if (P == WL_F16) load_spinor<P>(y, r + off, v.Vh, i);  // as stored
+        T nn = 0;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) nn = fma(y[c].re, y[c].re, fma(y[c].im, y[c].im, nn));
+        part[0] += (double)nn;
+    }
+    __shared__ double sh[32];
+    block_sum<1>(part, sh);
+    double tot[1];
+    if (grid_sum<1>(part, tot, red, rhs, gridDim.x, blockIdx.x, sh)) {
+        Scal& S = sc[rhs];
+        S.rr[0] = S.rr[2] = S.rh2 = tot[0];
+        S.rr[1] = 0.0;
+        S.rho_prev[0] = S.alpha[0] = S.omega[0] = 1.0;
+        S.rho_prev[1] = S.alpha[1] = S.omega[1] = 0.0;
+        S.fresh = 1;
+        restart_scalars(S);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -537,6 +580,7 @@ static int run_chunk_impl(wl_gauge g, Workspace* w, int nrhs, int k, bool use_gr
 int residual64(wl_gauge g, Workspace* w, int nrhs, cudaStream_t s)
 {
     const size_t hb = w->hb64;
+    w->rsrc = w->rhi;
     if (w->eo) {
         HopLaunch h1;
         h1.prec = w->outer;
@@ -673,8 +717,8 @@ int read_norms(Workspace* w, int nrhs, cudaStream_t s)
     return WL_OK;
 }
 
-// Begin an inner solve for the masked rhs: r = r_hi (converted), rhat = r,
-// p = v = x_lo = 0, fresh scalars with the given targets.
+// Begin an inner solve for the masked rhs: r = rhat = the outer residual
+// (converted), p = v = x_lo = 0, fresh scalars with the given targets.
 int inner_start(wl_gauge g, Workspace* w, int nrhs, const double* target2,
                        double delta2, cudaStream_t s)
 {
@@ -696,15 +740,21 @@ int inner_start(wl_gauge g, Workspace* w, int nrhs, const double* target2,
     // them is current after the last read-back)
     WL_CUDA(cudaMemcpyAsync(w->sc, w->sc_h, sizeof(Scal) * nrhs, cudaMemcpyHostToDevice, s));
     WL_TRY(upload_mask(w, nrhs, s));
-    WL_TRY(launch_convert(g, P, w->r, w->outer, w->rhi, w->nhalf, nrhs, w->mask, s));
-    WL_TRY(launch_convert(g, P, w->rh, P, w->r, w->nhalf, nrhs, w->mask, s));
-    WL_TRY(launch_zero(g, P, w->p, w->nhalf, nrhs, w->mask, s));
-    WL_TRY(launch_zero(g, P, w->v, w->nhalf, nrhs, w->mask, s));
-    WL_TRY(launch_zero(g, w->xlo_prec, w->xlo, w->nhalf, nrhs, w->mask, s));
-    WL_TRY(launch_cdot(g, P, w->rh, w->r, w->nhalf, nrhs, w->sc[0].rr, kScalStride, w->mask, s));
-    init_scal_kernel<<<(nrhs + 63) / 64, 64, 0, s>>>(w->sc, w->mask, nrhs, 1);
-    WL_CHECK_LAUNCH(0.0);
-    return WL_OK;
+    const Vec2 v = vec_of(g, P, w->nhalf), vs = vec_of(g, w->outer, w->nhalf);
+    return dispatch_prec(P, [&](auto pc) -> int {
+        constexpr int PP = decltype(pc)::value;
+        auto go = [&](auto* kernel) -> int {
+            const int vb = vec_block(w->nhalf * g->geo.Vh, g->num_sms);
+            const int resident = (resident_grid((const void*)kernel, vb, 0) + nrhs - 1) / nrhs;
+            const int blocks = (int)std::min<long long>((w->nhalf * g->geo.Vh + vb - 1) / vb, resident);
+            kernel<<<dim3((unsigned)blocks, (unsigned)nrhs), vb, 0, s>>>((char*)w->r, (char*)w->rh, v, (const char*)w->rsrc,
+                                                                          vs, w->mask, w->sc, g->red);
+            WL_CHECK_LAUNCH((double)(vs.hb + 2 * v.hb) * w->nhalf * nrhs);
+            return WL_OK;
+        };
+        if (w->outer == WL_F64) return go(round_start_kernel<PP, WL_F64>);
+        return go(round_start_kernel<PP, WL_DF64>);
+    });
 }
 
 // Reliable update for the masked rhs: x_hi += x_lo, x_lo = 0, r_hi = b' - A x_hi,
@@ -714,12 +764,13 @@ int reliable_update(wl_gauge g, Workspace* w, int nrhs, cudaStream_t s)
     const int P = w->inner;
     WL_TRY(upload_mask(w, nrhs, s));
     WL_TRY(launch_accum_hi(g, w->outer, w->xhi, w->xlo_prec, w->xlo, w->nhalf, nrhs, w->mask, s,
-                           full_rs(w)));
+                           full_rs(w), w->x_zero));
+    w->x_zero = false;
     WL_TRY(launch_zero(g, w->xlo_prec, w->xlo, w->nhalf, nrhs, w->mask, s));
     WL_TRY(residual64(g, w, nrhs, s));
-    WL_TRY(launch_convert(g, P, w->r, w->outer, w->rhi, w->nhalf, nrhs, w->mask, s));
+    WL_TRY(launch_convert(g, P, w->r, w->outer, w->rsrc, w->nhalf, nrhs, w->mask, s));
     WL_TRY(launch_cdot(g, P, w->rh, w->r, w->nhalf, nrhs, w->sc[0].rr, kScalStride, w->mask, s));
-    init_scal_kernel<<<(nrhs + 63) / 64, 64, 0, s>>>(w->sc, w->mask, nrhs, 0);
+    restart_scal_kernel<<<(nrhs + 63) / 64, 64, 0, s>>>(w->sc, w->mask, nrhs);
     WL_CHECK_LAUNCH(0.0);
     return WL_OK;
 }
@@ -828,7 +879,7 @@ int SolveState::begin_issue(wl_gauge g_, double* x, const double* b, int nrhs_, 
         WL_TRY(field_to_internal(g, w->xhi, xd, 0, w->outer, nrhs, s, 2 * (long long)hb64));
         WL_TRY(field_to_internal(g, (char*)w->xhi + hb64, xd, 1, w->outer, nrhs, s, 2 * (long long)hb64));
     }
-    if (!prm->use_x0) WL_CUDA(cudaMemsetAsync(w->xhi, 0, 2 * hb64 * nrhs, s));
+    w->x_zero = !prm->use_x0;
     // ||b||^2 over the full lattice, into the second set of norm slots
     WL_TRY(launch_cdot(g, WL_F64, w->b64, w->b64, 2, nrhs, w->nrm + 3 * nrhs, 3, nullptr, s));
     if (w->bout != w->b64)  // b in the outer precision
@@ -864,7 +915,7 @@ int SolveState::begin_issue(wl_gauge g_, double* x, const double* b, int nrhs_, 
         WL_TRY(upload_mask(w, nrhs, s));
         WL_TRY(residual64(g, w, nrhs, s));
     } else {  // x = 0: r = b' exactly, no FP64 matrix apply needed
-        WL_CUDA(cudaMemcpyAsync(w->rhi, w->bp, w->vb64 * nrhs, cudaMemcpyDeviceToDevice, s));
+        w->rsrc = w->bp;
         WL_TRY(launch_cdot(g, w->outer, w->bp, w->bp, w->nhalf, nrhs, w->nrm, 3, nullptr, s));
     }
     WL_CUDA(cudaMemcpyAsync(w->nrm_h, w->nrm, sizeof(double) * 6 * nrhs, cudaMemcpyDeviceToHost, s));
@@ -1063,10 +1114,12 @@ int SolveState::finish_round_issue(bool* pending)
         WL_TRY(upload_mask(w, nrhs, s));
         WL_TRY(launch_zero(g, w->xlo_prec, w->xlo, nh, nrhs, w->mask, s));
     }
-    for (int k = 0; k < nrhs; ++k) w->mask_h[k] = part[k];
+    // (x_lo holds nothing before a round's first iteration)
+    for (int k = 0; k < nrhs; ++k) w->mask_h[k] = part[k] && w->sc_h[k].iters > iters_before[k];
     WL_TRY(upload_mask(w, nrhs, s));
     WL_TRY(launch_accum_hi(g, w->outer, w->xhi, w->xlo_prec, w->xlo, nh, nrhs, w->mask, s,
-                           full_rs(w)));
+                           full_rs(w), w->x_zero));
+    w->x_zero = false;
     // a right-hand side whose inner solve just reached the final goal goes
     // straight to the true-residual check; the others need the FP64 residual
     int need = 0;
@@ -1122,6 +1175,10 @@ int SolveState::finalize(bool* retry_out)
 int SolveState::finalize_issue()
 {
     const size_t hb64 = w->hb64;
+    if (w->x_zero) {  // no right-hand side was iterated
+        WL_CUDA(cudaMemsetAsync(w->xhi, 0, 2 * hb64 * nrhs, s));
+        w->x_zero = false;
+    }
     if (w->x64 != w->xhi)  // the solution in FP64 (the even half for even-odd solves)
         WL_TRY(launch_convert(g, WL_F64, w->x64, w->outer, w->xhi, w->nhalf, nrhs, nullptr, s,
                               full_rs(w), full_rs(w)));

@@ -27,6 +27,8 @@ struct Scal {
     int iters;
     int flags;
     int want_update;
+    int fresh;          // no iteration of this round yet: p, v and x_lo hold nothing
+    int pad;
 };
 
 enum { FLAG_CONVERGED = 1, FLAG_BREAKDOWN = 2, FLAG_NAN = 4, FLAG_MAXITER = 8 };
@@ -53,6 +55,8 @@ struct Workspace {
     // is b in the outer precision (aliases b64 and xhi when the outer is FP64)
     double *b64 = nullptr, *bp = nullptr, *xhi = nullptr, *rhi = nullptr, *tmp64 = nullptr;
     double *bout = nullptr, *x64 = nullptr;
+    double* rsrc = nullptr;  // the outer residual a round starts from: bp (x0 = 0) or rhi
+    bool x_zero = false;     // x is still 0 and xhi not written: the first accumulation sets it
     Scal* sc = nullptr;
     Scal* sc_h = nullptr;  // pinned
     int* mask = nullptr;
@@ -120,11 +124,17 @@ __device__ __forceinline__ cx<double> safe_omega(const Scal& S)
     return {S.st[0] / S.st[2], -S.st[1] / S.st[2]};  // (t, s)/(t, t) = conj((s, t))/||t||^2
 }
 
-// p = r + beta (p - omega v)
+// p = r + beta (p - omega v); fresh: p = r (a round starts from p = v = 0)
 template <int P>
 __device__ __forceinline__ void p_update_site(char* p, const char* r, const char* v, long long Vh,
-                                              long long i, const double (&c)[4])
+                                              long long i, const double (&c)[4], bool fresh)
 {
+    if (fresh) {
+        cx<typename Prec<P>::real> rr[12];
+        load_spinor<P>(rr, r, Vh, i);
+        store_spinor<P>(p, Vh, i, rr);
+        return;
+    }
     using T = typename Prec<P>::real;
     const cx<T> beta = {(T)c[0], (T)c[1]}, om = {(T)c[2], (T)c[3]};
     cx<T> pp[12], rr[12], vv[12];
@@ -151,13 +161,14 @@ __device__ __forceinline__ void s_update_site(char* s, const char* r, const char
     store_spinor<P>(s, Vh, i, rr);
 }
 
-// x += alpha p + omega s;  r = s - omega t;  part = (rhat, r), ||r||^2 of the
-// stored (rounded) r, so rho matches what the next p update reads
+// x += alpha p + omega s (fresh: x = alpha p + omega s);  r = s - omega t;
+// part = (rhat, r), ||r||^2 of the stored (rounded) r, so rho matches what the
+// next p update reads
 template <int P, int PX>
 __device__ __forceinline__ void xr_update_site(char* x, char* r, const char* p, const char* s,
                                                const char* t, const char* rh, long long Vh,
                                                long long i, const double (&dc)[4],
-                                               typename Prec<P>::real (&part)[3])
+                                               typename Prec<P>::real (&part)[3], bool fresh)
 {
     using T = typename Prec<P>::real;
     using TX = typename Prec<PX>::real;
@@ -167,7 +178,12 @@ __device__ __forceinline__ void xr_update_site(char* x, char* r, const char* p, 
     load_spinor<P>(ss, s, Vh, i);
     {
         cx<TX> xx[12];
-        load_spinor<PX>(xx, x, Vh, i);
+        if (fresh) {
+#pragma unroll
+            for (int c = 0; c < 12; ++c) xx[c] = {(TX)0, (TX)0};
+        } else {
+            load_spinor<PX>(xx, x, Vh, i);
+        }
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
             const cx<T> d = al * pp[c] + om * ss[c];
@@ -210,6 +226,7 @@ __device__ __forceinline__ void advance_scalars(Scal& S, const double (&tot)[3],
     S.rr[1] = tot[1];
     S.rr[2] = tot[2];
     S.iters += 1;
+    S.fresh = 0;
     const bool stepped = (dc[0] != 0.0 || dc[1] != 0.0);
     const bool omega0 = (dc[2] == 0.0 && dc[3] == 0.0);
     if (!isfinite(tot[0]) || !isfinite(tot[1]) || !isfinite(tot[2])) {
