@@ -259,12 +259,12 @@ __device__ __forceinline__ void dd_hop_site(cx<typename Prec<P>::real> (&acc)[12
     using T = typename Prec<P>::real;
     const long long Vh = A.g.Vh;
     if constexpr (LF == 3) {
-        FxSum<3> Q;
-        DDFxSrc<HALO> src{{in, Vh, nb, links, Vh, i, 0}, A, remote, halo, f};
+        FxSum Q;
+        DDFxSrc<HALO> src{{in, Vh, nb, links, Vh, i}, A, remote, halo, f};
         fx_sum<DAG>(Q, src);
         const char* hl[6] = {halo[1][0], halo[1][1], halo[2][0], halo[2][1], halo[3][0], halo[3][1]};
         const long long fs[3] = {A.fs[1], A.fs[2], A.fs[3]}, fi[3] = {f[1], f[2], f[3]};
-        fx_finish<DAG>(acc, Q, links, Vh, i, 0, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
+        fx_finish<DAG>(acc, Q, links, Vh, i, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
             if (HALO && ((remote >> d) & 1)) {  // (never the x hops d = 0, 1)
                 float unused;
                 load_half<WL_F64>(h0, h1, unused, hl[d - 2], fs[(d >> 1) - 1], fi[(d >> 1) - 1]);

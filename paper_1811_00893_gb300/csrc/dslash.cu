@@ -99,8 +99,11 @@ static const int kPipeShape = 16;
 // Single-RHS reducing launches: block size (grid of resident blocks), or
 // kFullGrid + block size (full grid and a finishing launch).
 static const int kFullGrid = 1000;
-// Single-RHS FP64 Wilson launches: three threads per site (hop_rows_kernel).
+// Single-RHS FP64 Wilson launches: several threads per site (hop_rows_kernel, hop_fx_rows_kernel).
 static const int kRowsShape = 2000;
+// Largest launch (output sites x right-hand sides) the autotuner times it for
+// with fixed-point links: 16^3 x 32 and up take one thread per site everywhere.
+static const long long kRowsMost = 65536;
 // Multi-RHS launches of the wide types: kPerRhs + block size = the single-RHS
 // kernel with one grid row per right-hand side (grid.y), links read once per
 // right-hand side (these launches are bound by arithmetic, not by bytes);
@@ -131,12 +134,13 @@ static int launch_shape(const HopLaunch& h, int lf, HopArgs& A, int nrhs, int sh
     A.blocks_per_parity = (int)bpp;
     A.nparity = h.nparity;
     unsigned gx = (unsigned)(bpp * h.nparity);
-    if (!multi && shape == kRowsShape) {
-        A.blocks_per_parity = (int)((A.g.Vh + kRowSites - 1) / kRowSites);
-        A.partials_only = h.dot ? 1 : 0;
+    if (shape == kRowsShape) {  // (several right-hand sides: fixed point only)
+        const int sites = lf == 3 ? kFxRowSites : kRowSites;
+        A.blocks_per_parity = (int)((A.g.Vh + sites - 1) / sites);
+        A.partials_only = h.dot && lf != 3 ? 1 : 0;  // (fixed point: added by the last block)
         gx = (unsigned)((long long)A.blocks_per_parity * h.nparity);
-        with_variant(h, lf, [&](auto K) { K.rows(h.dagger != 0, h.dot, A, dim3(gx, 1), s); });
-        if (h.dot)
+        with_variant(h, lf, [&](auto K) { K.rows(h.dagger != 0, h.dot, A, dim3(gx, (unsigned)nrhs), s); });
+        if (A.partials_only)
             return launch_finish_slots(A.red.partial, (long long)A.red.max_blocks * 3, (int)gx, 1, A.dot_out,
                                        A.dot_stride, A.active, A.active_stride, s);
     } else if (!multi) {
@@ -229,13 +233,16 @@ static int tuned_shape(wl_gauge g, const HopLaunch& h, int lf, HopArgs& A, int n
             return WL_OK;
         }
     }
-    if (multi && lf == 3) return WL_OK;  // one form
     if (!autotune_enabled() || is_capturing(s)) return WL_OK;
     std::vector<int> cand;
-    if (lf == 3) {  // (one site per thread in kFxBlock-thread blocks, or kRowsShape)
-        cand = {kFxBlock};
-        if (h.dot) cand.push_back(kFullGrid + kFxBlock);
-        if (rows_allowed(h, lf)) cand.push_back(kRowsShape);
+    if (lf == 3) {  // one site per thread in kFxBlock-thread blocks, or kRowsShape where that has few blocks per SM
+        cand = {multi ? kPerRhs + kFxBlock : kFxBlock};
+        if (h.dot && !multi) cand.push_back(kFullGrid + kFxBlock);
+        if (rows_allowed(h, lf) && g->geo.Vh * h.nparity * nrhs <= kRowsMost) cand.push_back(kRowsShape);
+        if (cand.size() == 1) {
+            *shape = cand[0];
+            return WL_OK;
+        }
     } else if (multi) {
         for (int l : {1, 2, 4, 8})
             if (l <= nrhs) cand.push_back(l);
@@ -303,7 +310,7 @@ static int launch_hop_chunk(wl_gauge g, const HopLaunch& h, int lf, HopArgs A, i
 {
     const bool multi = nrhs > 1;
     if (h.dot) {  // sized for the smallest tile any candidate shape uses
-        const long long most = ((g->geo.Vh + 31) / 32) * h.nparity;
+        const long long most = ((g->geo.Vh + kFxRowSites - 1) / kFxRowSites) * h.nparity;
         WL_TRY(ensure_red(g, nrhs, most));
     }
     A.red = g->red;

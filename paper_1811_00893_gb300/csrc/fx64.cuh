@@ -51,19 +51,17 @@ __device__ __forceinline__ double fx_join(int h, int l)
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
 __device__ __forceinline__ long long fx_mul(int a, int b) { return (long long)a * b; }
 
-// NR colour rows of the site sum: s[(spin * NR + row) * 2 + (0: re, 1: im)]
-template <int NR>
+// The site sum: s[(spin * 3 + colour row) * 2 + (0: re, 1: im)]
 struct FxSum {
-    long long s[8 * NR];
+    long long s[24];
     int e;     // biased exponent of the units
     bool bad;  // this site needs fx_site_general
 };
 
-template <int NR>
-__device__ __forceinline__ void fx_clear(FxSum<NR>& S)
+__device__ __forceinline__ void fx_clear(FxSum& S)
 {
 #pragma unroll
-    for (int k = 0; k < 8 * NR; ++k) S.s[k] = 0;
+    for (int k = 0; k < 24; ++k) S.s[k] = 0;
     S.e = kFxMinExp;
     S.bad = false;
 }
@@ -94,8 +92,7 @@ struct FxHalf {
 };
 
 // Convert the half spinor (h0, h1), raising Q's exponent first if it exceeds it.
-template <int NR>
-__device__ __forceinline__ void fx_convert(FxSum<NR>& Q, FxHalf& X, const cx<double> (&h0)[3], const cx<double> (&h1)[3])
+__device__ __forceinline__ void fx_convert(FxSum& Q, FxHalf& X, const cx<double> (&h0)[3], const cx<double> (&h1)[3])
 {
     unsigned hw[12], lw[12];
 #pragma unroll
@@ -128,7 +125,7 @@ __device__ __forceinline__ void fx_convert(FxSum<NR>& Q, FxHalf& X, const cx<dou
         if (by > 0) {
             const long long half = 1LL << (by - 1);
 #pragma unroll
-            for (int k = 0; k < 8 * NR; ++k) Q.s[k] = (Q.s[k] + half) >> by;
+            for (int k = 0; k < 24; ++k) Q.s[k] = (Q.s[k] + half) >> by;
         }
 #pragma unroll
         for (int q = 0; q < 12; ++q) up[q] += (E - Q.e) << 20;
@@ -139,8 +136,7 @@ __device__ __forceinline__ void fx_convert(FxSum<NR>& Q, FxHalf& X, const cx<dou
         const unsigned mh = (hw[q] & 0xfffffu) | 0x100000u;
         // the 53-bit significand 7 bits up, then down by the exponent difference
         // (zeros and subnormals: by 63, to 0)
-        unsigned long long y = (unsigned long long)lw[q] * 128u;
-        y += (unsigned long long)(mh * 128u) << 32;
+        unsigned long long y = ((unsigned long long)__funnelshift_l(lw[q], mh, 7) << 32) | (lw[q] << 7);
         y >>= min((unsigned)up[q] >> 20, 63u);
         const int sg = ((int)hw[q] >> 31) | 1;
         X.xh[q] = (int)(unsigned)(y >> 32) * sg;
@@ -152,8 +148,7 @@ __device__ __forceinline__ void fx_convert(FxSum<NR>& Q, FxHalf& X, const cx<dou
 // converted half spinor X.  X holds S (h0, h1) for the projector 1 + S gamma_mu,
 // so rows 2 and 3 take it as it is, and rows 0 and 1 are summed with the sign S
 // (the sign of the present pass, see fx_sum).
-template <int NR>
-__device__ __forceinline__ void fx_row(FxSum<NR>& Q, const FxHalf& X, const int4 (&w)[3], int r, int mu)
+__device__ __forceinline__ void fx_row(FxSum& Q, const FxHalf& X, const int4 (&w)[3], int r, int mu)
 {
     long long R[4];  // u0.re, u0.im, u1.re, u1.im
 #pragma unroll
@@ -182,7 +177,7 @@ __device__ __forceinline__ void fx_row(FxSum<NR>& Q, const FxHalf& X, const int4
         R[2 * j] = A + (B >> 31);
         R[2 * j + 1] = C + (D >> 31);
     }
-    long long *s0 = Q.s + 2 * r, *s1 = s0 + 2 * NR, *s2 = s1 + 2 * NR, *s3 = s2 + 2 * NR;
+    long long *s0 = Q.s + 2 * r, *s1 = s0 + 6, *s2 = s1 + 6, *s3 = s2 + 6;
     fx_add_ik<0>(s0, R[0], R[1]);
     fx_add_ik<0>(s1, R[2], R[3]);
     if (mu & 1) {
@@ -202,11 +197,10 @@ __device__ __forceinline__ void fx_row(FxSum<NR>& Q, const FxHalf& X, const int4
     }
 }
 
-template <int NR>
-__device__ __forceinline__ void fx_negate_upper(FxSum<NR>& Q)
+__device__ __forceinline__ void fx_negate_upper(FxSum& Q)
 {
 #pragma unroll
-    for (int k = 0; k < 4 * NR; ++k) Q.s[k] = -Q.s[k];
+    for (int k = 0; k < 12; ++k) Q.s[k] = -Q.s[k];
 }
 
 // S times the projected half spinor of (1 + S gamma_mu), S = sg = 1 or -1, from
@@ -260,9 +254,9 @@ __device__ __forceinline__ int fx_order(int k) { return 2 * (k & 3) + (k >> 2); 
 // direction a uniform branch where its spin structure enters.  src gives
 // hop fx_order(k) its data:
 //   half(k, mu, sg, h0, h1)  sg times the projected half spinor
-//   link(k, r, w)            row a0 + r of the link
-template <bool DAG, int NR, typename Src>
-__device__ __forceinline__ void fx_sum(FxSum<NR>& Q, Src& src)
+//   link(k, r, w)            row r of the link
+template <bool DAG, typename Src>
+__device__ __forceinline__ void fx_sum(FxSum& Q, Src& src)
 {
     fx_clear(Q);
 #pragma unroll 1
@@ -276,7 +270,7 @@ __device__ __forceinline__ void fx_sum(FxSum<NR>& Q, Src& src)
             fx_convert(Q, X, h0, h1);
         }
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
+        for (int r = 0; r < 3; ++r) {
             int4 w[3];
             src.link(k, r, w);
             fx_row(Q, X, w, r, mu);
@@ -287,7 +281,7 @@ __device__ __forceinline__ void fx_sum(FxSum<NR>& Q, Src& src)
     // cancels between hops that add and hops that subtract, except in the real part of
     // row 2, which adds all eight
 #pragma unroll
-    for (int r = 0; r < NR; ++r) Q.s[2 * (2 * NR + r)] += 4;
+    for (int r = 0; r < 3; ++r) Q.s[2 * (6 + r)] += 4;
 }
 
 // s 2^(e-1023-55) rounded to nearest, ties to even, by integer operations
@@ -371,25 +365,20 @@ __device__ __noinline__ void fx_site_general(double (&out)[24], const void* link
     }
 }
 
-// Rows a0 .. a0 + NR - 1 of the site sum as FP64: acc[spin * 3 + r] for row a0 + r
-template <bool DAG, int NR, typename F>
-__device__ __forceinline__ void fx_finish(cx<double> (&acc)[12], const FxSum<NR>& S, const void* links, long long lVh,
-                                          long long li, int a0, F half)
+// acc = the site sum as FP64
+template <bool DAG, typename F>
+__device__ __forceinline__ void fx_finish(cx<double> (&acc)[12], const FxSum& S, const void* links, long long lVh,
+                                          long long li, F half)
 {
     if (S.bad || S.e == kFxMinExp) {  // (nothing above 2^-953: zeros, or too small for fixed point)
         double g[24];
         fx_site_general<DAG>(g, links, lVh, li, half);
 #pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-            for (int r = 0; r < NR; ++r) acc[3 * sp + r] = {g[2 * (3 * sp + a0 + r)], g[2 * (3 * sp + a0 + r) + 1]};
+        for (int c = 0; c < 12; ++c) acc[c] = {g[2 * c], g[2 * c + 1]};
         return;
     }
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int r = 0; r < NR; ++r)
-            acc[3 * sp + r] = {fx_value(S.s[2 * (NR * sp + r)], S.e), fx_value(S.s[2 * (NR * sp + r) + 1], S.e)};
+    for (int c = 0; c < 12; ++c) acc[c] = {fx_value(S.s[2 * c], S.e), fx_value(S.s[2 * c + 1], S.e)};
 }
 
 // The plain-FP64 path's half spinor of hop d from the local neighbour at n
@@ -420,7 +409,6 @@ struct FxDirect {
     const void* links;
     long long lVh;
     long long li;
-    int a0;
 
     __device__ __forceinline__ void half(int k, int mu, double sg, cx<double> (&h0)[3], cx<double> (&h1)[3])
     {
@@ -430,22 +418,21 @@ struct FxDirect {
     }
     __device__ __forceinline__ void link(int k, int r, int4 (&w)[3])
     {
-        const int4* p = (const int4*)links + (fx_order(k) * 9 + 3 * (a0 + r)) * lVh + li;
+        const int4* p = (const int4*)links + (fx_order(k) * 9 + 3 * r) * lVh + li;
 #pragma unroll
         for (int c = 0; c < 3; ++c) w[c] = p[c * lVh];
     }
 };
 
-// acc = H_{p,1-p} in at the output site whose neighbours are nb: rows a0 ..
-// a0 + NR - 1 (hop_site for LF = 3; hop_rows_kernel takes one row per thread).
-template <bool DAG, int NR>
+// acc = H_{p,1-p} in at the output site whose neighbours are nb (hop_site for LF = 3)
+template <bool DAG>
 __device__ __forceinline__ void fx_site(cx<double> (&acc)[12], const int (&nb)[8], long long Vh, const void* in,
-                                        const void* links, long long lVh, int li, int a0)
+                                        const void* links, long long lVh, int li)
 {
-    FxSum<NR> S;
-    FxDirect src{in, Vh, nb, links, lVh, li, a0};
+    FxSum S;
+    FxDirect src{in, Vh, nb, links, lVh, li};
     fx_sum<DAG>(S, src);
-    fx_finish<DAG>(acc, S, links, lVh, li, a0, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
+    fx_finish<DAG>(acc, S, links, lVh, li, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
         fx_general_local<DAG>(d, h0, h1, in, Vh, fx_pick(nb, d));
     });
 }
@@ -527,14 +514,225 @@ template <bool DAG>
 __device__ __forceinline__ void fx_site_staged(cx<double> (&acc)[12], const int (&nb)[8], long long Vh, const char* in,
                                                const char* links, long long lVh, int li, int4* slot)
 {
-    FxSum<3> S;
+    FxSum S;
     FxStaged src{slot, in, Vh, links + (unsigned)li * 16u, lVh};
     src.start(nb);
     fx_sum<DAG>(S, src);
     cp_async_wait<0>();
-    fx_finish<DAG>(acc, S, links, lVh, li, 0, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
+    fx_finish<DAG>(acc, S, links, lVh, li, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
         fx_general_local<DAG>(d, h0, h1, in, Vh, src.neighbour(d));
     });
+}
+
+// ---------------------------------------------------------------------------
+// Small lattices, where a thread per site leaves the SMs with a warp or two and
+// the time is one thread's dependent instructions: six threads per site, one
+// for each of the rows j = 0, 1 of the half spinors and each colour row r.
+// Lanes l and l + 16 of a warp hold j = 0 and 1 of the same site and colour row.
+// The sums are fx_sum's, bit for bit: the two threads agree on e at every
+// hop, and join their parts of spin rows 2 and 3 before they are shifted.
+// ---------------------------------------------------------------------------
+
+// Spin row j in s, this thread's parts of spin rows 3 - j and 2 + j in a and b (re, im)
+struct FxPart {
+    long long s[2], a[2], b[2];
+    int e;
+    bool bad;
+};
+
+__device__ __forceinline__ long long fx_partner(long long v) { return __shfl_xor_sync(0xffffffffu, v, 16); }
+
+// fx_convert for one projected row (colour x (re, im)); whole warps call it
+__device__ __forceinline__ void fx_convert_row(FxPart& Q, int (&xh)[6], int (&xl)[6], const cx<double> (&h)[3])
+{
+    unsigned hw[6], lw[6];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        hw[2 * c] = (unsigned)__double2hiint(h[c].re);
+        lw[2 * c] = (unsigned)__double2loint(h[c].re);
+        hw[2 * c + 1] = (unsigned)__double2hiint(h[c].im);
+        lw[2 * c + 1] = (unsigned)__double2loint(h[c].im);
+    }
+    int up[6], any = 0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        up[q] = (int)((((unsigned)Q.e << 20) | 0xfffffu) - (hw[q] & 0x7fffffffu));
+        any |= up[q];
+    }
+    if (__any_sync(0xffffffffu, any < 0)) {
+        unsigned top = 0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) top = max(top, hw[q] & 0x7fffffffu);
+        top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
+        int E = (int)(top >> 20);
+        if (E > Q.e) {
+            E += Q.e == kFxMinExp ? 1 : 0;
+            if (E > kFxMaxExp) {
+                Q.bad = true;
+                E = kFxMaxExp;  // (the sums are not used any more)
+            }
+        } else {
+            E = Q.e;  // another site's
+        }
+        const int by = min(E - Q.e, 62);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            Q.b[k] += fx_partner(Q.a[k]);
+            Q.a[k] = 0;
+            if (by > 0) {
+                const long long half = 1LL << (by - 1);
+                Q.s[k] = (Q.s[k] + half) >> by;
+                Q.b[k] = (Q.b[k] + half) >> by;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) up[q] += (E - Q.e) << 20;
+        Q.e = E;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        const unsigned mh = (hw[q] & 0xfffffu) | 0x100000u;
+        unsigned long long y = ((unsigned long long)__funnelshift_l(lw[q], mh, 7) << 32) | (lw[q] << 7);
+        y >>= min((unsigned)up[q] >> 20, 63u);
+        const int sg = ((int)hw[q] >> 31) | 1;
+        xh[q] = (int)(unsigned)(y >> 32) * sg;
+        xl[q] = (int)((unsigned)y >> 1) * sg;
+    }
+}
+
+// The sign that hop direction MU and row j give the neighbour's spin rows 2 and
+// 3 next to the projector's S: -1 for (y, 0) and (z, 1)
+template <int MU>
+__device__ __forceinline__ int fx_minus(int j)
+{
+    return MU == 1 ? j - 1 : MU == 2 ? -j : 0;
+}
+
+// One hop of direction MU: own spin row p of the neighbour, its row q = 3 - j
+// (MU = x, y) or 2 + j (z, t), row w of the link; sg as in fx_project.  The
+// projected row is S p + c q, c = i (x, z) or 1 (y, t) with the sign m; its
+// product enters spin row j, and spin row 3 - j or 2 + j with -i or 1 and m.
+template <int MU>
+__device__ __forceinline__ void fx_hop_row(FxPart& Q, const cx<double> (&p)[3], const cx<double> (&q)[3], const int4 (&w)[3],
+                                           int j, double sg)
+{
+    const int m = fx_minus<MU>(j);
+    auto flip = [=](double v) {  // v, or -v for m = -1
+        return __hiloint2double((int)((unsigned)__double2hiint(v) ^ ((unsigned)m & 0x80000000u)), __double2loint(v));
+    };
+    cx<double> h[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        cx<double> t = q[c];
+        if constexpr (MU == 1 || MU == 2) t = {flip(t.re), flip(t.im)};
+        if constexpr (MU == 0 || MU == 2) t = mul_i(t);
+        h[c] = {fma(sg, p[c].re, t.re), fma(sg, p[c].im, t.im)};
+    }
+    int H[6], L[6];
+    fx_convert_row(Q, H, L, h);
+    long long A = 0, B = 0, C = 0, D = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        A = fx_mad(w[k].x, H[2 * k], A);
+        A = fx_mad(-w[k].z, H[2 * k + 1], A);
+        B = fx_mad(w[k].x, L[2 * k], B);
+        B = fx_mad(w[k].y, H[2 * k], B);
+        B = fx_mad(-w[k].z, L[2 * k + 1], B);
+        B = fx_mad(-w[k].w, H[2 * k + 1], B);
+        C = fx_mad(w[k].x, H[2 * k + 1], C);
+        C = fx_mad(w[k].z, H[2 * k], C);
+        D = fx_mad(w[k].x, L[2 * k + 1], D);
+        D = fx_mad(w[k].y, H[2 * k + 1], D);
+        D = fx_mad(w[k].z, L[2 * k], D);
+        D = fx_mad(w[k].w, H[2 * k], D);
+    }
+    const long long re = A + (B >> 31), im = C + (D >> 31);
+    Q.s[0] += re;
+    Q.s[1] += im;
+    const long long mm = m;
+    if constexpr (MU == 0) {
+        Q.a[0] += im;
+        Q.a[1] -= re;
+    } else if constexpr (MU == 1) {
+        Q.a[0] += (re ^ mm) - mm;
+        Q.a[1] += (im ^ mm) - mm;
+    } else if constexpr (MU == 2) {
+        Q.b[0] += (im ^ mm) - mm;
+        Q.b[1] -= (re ^ mm) - mm;
+    } else {
+        Q.b[0] += re;
+        Q.b[1] += im;
+    }
+}
+
+// Colour row a of spin rows j (up) and 2 + j (down) of the site sum at li, j =
+// lane >> 4.  Every load of a hop is issued a hop ahead into registers.  Whole
+// warps call it.
+template <bool DAG>
+__device__ __forceinline__ void fx_site_row(cx<double>& up, cx<double>& down, const int (&nb)[8], long long Vh, const void* in,
+                                            const void* links, long long li, int a, int lane)
+{
+    const int j = lane >> 4;
+    FxPart Q;
+    Q.s[0] = Q.s[1] = Q.a[0] = Q.a[1] = Q.b[0] = Q.b[1] = 0;
+    Q.e = kFxMinExp;
+    Q.bad = false;
+    const double2* f = (const double2*)in + 3 * j * Vh;
+    const int4* l = (const int4*)links + 3 * a * Vh + li;
+    cx<double> p[3], q[3];
+    int4 w[3];
+    auto load = [&](int d, int n) {  // neighbour n through link d
+        const long long g = (d < 4 ? 9 - 6 * j : 6) * Vh;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 u = __ldg(f + c * Vh + n), v = __ldg(f + g + c * Vh + n);
+            p[c] = {u.x, u.y};
+            q[c] = {v.x, v.y};
+            w[c] = l[(d * 9 + c) * Vh];
+        }
+    };
+    load(0, nb[0]);
+#pragma unroll 1
+    for (int fb = 0; fb < 2; ++fb) {
+        const double sg = (fb == 0) != DAG ? -1.0 : 1.0;
+        auto hop = [&](auto mu) {
+            constexpr int MU = decltype(mu)::value;
+            cx<double> p0[3], q0[3];
+            int4 w0[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                p0[c] = p[c];
+                q0[c] = q[c];
+                w0[c] = w[c];
+            }
+            if constexpr (MU < 3) load(2 * MU + 2 + fb, fb ? nb[2 * MU + 3] : nb[2 * MU + 2]);
+            else if (fb == 0) load(1, nb[1]);
+            fx_hop_row<MU>(Q, p0, q0, w0, j, sg);
+        };
+        hop(std::integral_constant<int, 0>());
+        hop(std::integral_constant<int, 1>());
+        hop(std::integral_constant<int, 2>());
+        hop(std::integral_constant<int, 3>());
+        if (fb == 0 || DAG) {
+            Q.s[0] = -Q.s[0];
+            Q.s[1] = -Q.s[1];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) Q.b[k] += fx_partner(Q.a[k]);
+    Q.b[0] += j == 0 ? 4 : 0;  // (as fx_sum)
+    if (Q.bad || Q.e == kFxMinExp) {
+        double g[24];
+        fx_site_general<DAG>(g, links, Vh, li, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
+            fx_general_local<DAG>(d, h0, h1, in, Vh, fx_pick(nb, d));
+        });
+        const int c = 2 * (3 * j + a);
+        up = {g[c], g[c + 1]};
+        down = {g[c + 12], g[c + 13]};
+        return;
+    }
+    up = {fx_value(Q.s[0], Q.e), fx_value(Q.s[1], Q.e)};
+    down = {fx_value(Q.b[0], Q.e), fx_value(Q.b[1], Q.e)};
 }
 
 }  // namespace wl

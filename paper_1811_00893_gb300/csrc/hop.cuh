@@ -780,7 +780,7 @@ __device__ __forceinline__ void hop_site(cx<typename Prec<P>::real> (&acc)[12], 
         hop_site_loop<P, DAG>(acc, nb, Vh, in, links, lVh, li);
     } else if constexpr (LF == 3) {  // (the kernels that have shared memory for it call fx_site_staged)
         static_assert(P == WL_F64, "fixed-point links are FP64's");
-        fx_site<DAG, 3>(acc, nb, Vh, in, links, lVh, li, 0);
+        fx_site<DAG>(acc, nb, Vh, in, links, lVh, li);
     } else {
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = {(T)0, (T)0};

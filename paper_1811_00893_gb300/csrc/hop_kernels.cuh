@@ -316,15 +316,81 @@ __global__ void __launch_bounds__(kFxBlock, 8) hop_fx_kernel(const HopArgs A)
     }
 }
 
+// The same for small lattices, six threads per site (fx_site_row): 16 sites per
+// block, warp a the colour row a of them.  A thread has a sixth of a site's
+// products and a third of its conversions, and FP64 operations (64 clocks each
+// to a warp) are spread over all four schedulers of the SMs.  8^4 full D: three
+// threads per site 14.5 us, six 9.7 us; with its reductions (ncu) one thread
+// per site 27.5 us, six 16.1 us.
+static constexpr int kFxRowSites = 16, kFxRowBlock = 96;
+
+template <bool DAG, bool DOT>
+__global__ void __launch_bounds__(kFxRowBlock) hop_fx_rows_kernel(const HopArgs A)
+{
+    const int rhs = blockIdx.y;
+    if (A.active && A.active[rhs * A.active_stride] == 0) return;  // uniform per block
+    const int pidx = blockIdx.x / A.blocks_per_parity;
+    const int lane = threadIdx.x & 31, a = threadIdx.x >> 5, j = lane >> 4;
+    const int site = (blockIdx.x - pidx * A.blocks_per_parity) * kFxRowSites + (lane & 15);
+    const long long Vh = A.g.Vh;
+    const bool valid = site < Vh;
+    const int i = valid ? site : (int)Vh - 1;  // (whole warps: the partners exchange sums)
+    double part[3] = {0, 0, 0};
+    {
+        int nb[8];
+        neighbours(A.g, A.parity0 + pidx, i, nb);
+        cx<double> v[2];  // components (spin j, colour a) and (2 + j, a)
+        fx_site_row<DAG>(v[0], v[1], nb, Vh, A.in[pidx] + rhs * A.rs_in, A.links[pidx], i, a, lane);
+        if (valid) {  // epilogue, the operations of epilogue_ptrs on each component
+            auto at = [&](const char* q, long long rs) { return (const double2*)(q ? q + rhs * rs : nullptr); };
+            const double2 *x1 = at(A.x1[pidx], A.rs_x1), *x2 = at(A.x2[pidx], A.rs_x2), *w = at(A.w[pidx], A.rs_w);
+            double2* out = (double2*)(A.out[pidx] + rhs * A.rs_out);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const long long o = (3 * (j + 2 * s) + a) * Vh + i;
+                if (A.a != 1.0) v[s] = A.a * v[s];
+                if (x1) {
+                    const double2 t = x1[o];
+                    v[s] = v[s] + cx<double>{t.x, t.y};
+                }
+                if (x2) {
+                    const double2 t = x2[o];
+                    v[s] = v[s] + A.b1 * cx<double>{t.x, t.y};
+                }
+                out[o] = make_double2(v[s].re, v[s].im);
+                if (DOT) {
+                    if (w) {
+                        const double2 t = w[o];
+                        part[0] = fma(t.x, v[s].re, fma(t.y, v[s].im, part[0]));
+                        part[1] = fma(t.x, v[s].im, fma(-t.y, v[s].re, part[1]));
+                    }
+                    part[2] = fma(v[s].re, v[s].re, fma(v[s].im, v[s].im, part[2]));
+                }
+            }
+        }
+    }
+    if constexpr (DOT) {
+        __shared__ double sh[3 * 32];
+        warp_sum<3>(part);
+        block_sum_warps<3>(part, sh);
+        double tot[3];
+        if (grid_sum<3>(part, tot, A.red, rhs, gridDim.x, blockIdx.x, sh)) {
+            double* o = A.dot_out + (long long)rhs * A.dot_stride;
+            o[0] = tot[0];
+            o[1] = tot[1];
+            o[2] = tot[2];
+        }
+    }
+}
+
 // FP64 hopping term for small lattices, where one thread per site leaves
 // most SMs with less than a warp and the kernel's time is the latency of one
 // thread's dependent FP64 chain: three threads per output site, one colour
 // row a each (output components 3 s + a).  Each projects the full neighbour
 // spinors (the three rows read them from L1) and applies row a of every link,
 // a third of hop_kernel's chain per thread and no exchange between the three.
-// Every output component sees hop_kernel's operations in the same order (with
-// fixed-point links, hop_fx_kernel's; there one thread per site takes 20 us on
-// 8^4, three threads 14.6 us).
+// Every output component sees hop_kernel's operations in the same order.
+// (Links that do not fit fixed point; the others take hop_fx_rows_kernel.)
 // Block: kRowSites sites x 3 rows (thread t: row t / kRowSites); a reducing
 // launch leaves one partial per block for the finishing launch.  32 sites per
 // block spread an 8^4 lattice's 2 x 2,048 sites over 128 SMs: on small lattices
@@ -341,7 +407,7 @@ __device__ __forceinline__ void hop_row(cx<double> (&acc)[12], const char* in, l
     reconstruct<MU, S>(acc, 0, dot3(w[0], w[1], w[2], h0), dot3(w[0], w[1], w[2], h1));
 }
 
-template <bool DAG, bool DOT, int LF>
+template <bool DAG, bool DOT>
 __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A)
 {
     const int rhs = blockIdx.y;
@@ -357,22 +423,18 @@ __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A
         const char* in = A.in[pidx] + rhs * A.rs_in;
         const void* links = A.links[pidx];
         cx<double> acc[12];  // the rows of colour a at 0, 3, 6, 9
-        if constexpr (LF == 3) {
-            fx_site<DAG, 1>(acc, nb, Vh, in, links, Vh, i, a);
-        } else {
 #pragma unroll
-            for (int c = 0; c < 12; ++c) acc[c] = {0.0, 0.0};
-            constexpr int F = DAG ? +1 : -1;  // forward projector sign
-            constexpr int B = -F;
-            hop_row<0, 0, F>(acc, in, Vh, nb[0], links, i, a);
-            hop_row<1, 0, B>(acc, in, Vh, nb[1], links, i, a);
-            hop_row<2, 1, F>(acc, in, Vh, nb[2], links, i, a);
-            hop_row<3, 1, B>(acc, in, Vh, nb[3], links, i, a);
-            hop_row<4, 2, F>(acc, in, Vh, nb[4], links, i, a);
-            hop_row<5, 2, B>(acc, in, Vh, nb[5], links, i, a);
-            hop_row<6, 3, F>(acc, in, Vh, nb[6], links, i, a);
-            hop_row<7, 3, B>(acc, in, Vh, nb[7], links, i, a);
-        }
+        for (int c = 0; c < 12; ++c) acc[c] = {0.0, 0.0};
+        constexpr int F = DAG ? +1 : -1;  // forward projector sign
+        constexpr int B = -F;
+        hop_row<0, 0, F>(acc, in, Vh, nb[0], links, i, a);
+        hop_row<1, 0, B>(acc, in, Vh, nb[1], links, i, a);
+        hop_row<2, 1, F>(acc, in, Vh, nb[2], links, i, a);
+        hop_row<3, 1, B>(acc, in, Vh, nb[3], links, i, a);
+        hop_row<4, 2, F>(acc, in, Vh, nb[4], links, i, a);
+        hop_row<5, 2, B>(acc, in, Vh, nb[5], links, i, a);
+        hop_row<6, 3, F>(acc, in, Vh, nb[6], links, i, a);
+        hop_row<7, 3, B>(acc, in, Vh, nb[7], links, i, a);
         // epilogue (as epilogue_ptrs, on this thread's four components)
         auto at = [&](const char* q, long long rs) -> const double2* {
             return q ? (const double2*)(q + rhs * rs) : nullptr;
@@ -433,7 +495,7 @@ struct HopKernels {
     static void pipe(int prec, bool dagger, bool dot, const HopArgs& A, int nrhs, int ntiles, dim3 grid,
                      dim3 block, size_t smem, cudaStream_t s);
     static const void* pipe_kernel(int prec, bool dagger, bool dot);
-    // three threads per site (FP64, CL = 0, LF = 0 or 3), kRowSites sites per block
+    // small lattices (FP64, CL = 0): three threads per site (LF = 0, kRowSites sites per block) or six (LF = 3, kFxRowSites)
     static void rows(bool dagger, bool dot, const HopArgs& A, dim3 grid, cudaStream_t s);
     // the reducing single-RHS kernel (for occupancy queries)
     static const void* reducing(int prec, bool dagger);
@@ -554,14 +616,22 @@ void HopKernels<CL, LF>::multi(int prec, bool dagger, bool dot, const HopArgs& A
 template <int CL, int LF>
 void HopKernels<CL, LF>::rows(bool dagger, bool dot, const HopArgs& A, dim3 grid, cudaStream_t s)
 {
-    if constexpr (CL == kClNone && (LF == 0 || LF == 3)) {
+    if constexpr (CL == kClNone && LF == 3) {
+        if (dagger) {
+            if (dot) hop_fx_rows_kernel<true, true><<<grid, kFxRowBlock, 0, s>>>(A);
+            else hop_fx_rows_kernel<true, false><<<grid, kFxRowBlock, 0, s>>>(A);
+        } else {
+            if (dot) hop_fx_rows_kernel<false, true><<<grid, kFxRowBlock, 0, s>>>(A);
+            else hop_fx_rows_kernel<false, false><<<grid, kFxRowBlock, 0, s>>>(A);
+        }
+    } else if constexpr (CL == kClNone && LF == 0) {
         const int block = 3 * kRowSites;
         if (dagger) {
-            if (dot) hop_rows_kernel<true, true, LF><<<grid, block, 0, s>>>(A);
-            else hop_rows_kernel<true, false, LF><<<grid, block, 0, s>>>(A);
+            if (dot) hop_rows_kernel<true, true><<<grid, block, 0, s>>>(A);
+            else hop_rows_kernel<true, false><<<grid, block, 0, s>>>(A);
         } else {
-            if (dot) hop_rows_kernel<false, true, LF><<<grid, block, 0, s>>>(A);
-            else hop_rows_kernel<false, false, LF><<<grid, block, 0, s>>>(A);
+            if (dot) hop_rows_kernel<false, true><<<grid, block, 0, s>>>(A);
+            else hop_rows_kernel<false, false><<<grid, block, 0, s>>>(A);
         }
     }
 }

@@ -96,6 +96,29 @@ __device__ __forceinline__ long long split_index(const Vec2& v, long long j, lon
     return j - h * v.Vh;
 }
 
+// Threads per site of the updates below and their components: FP64 splits a
+// site over four (solver.cuh, p_update_part).
+template <int P>
+struct VecSplit {
+    static constexpr int threads = P == WL_F64 ? 4 : 1;
+};
+static int vec_split(int prec) { return prec == WL_F64 ? VecSplit<WL_F64>::threads : 1; }
+
+// Element e of n site elements x VecSplit threads: returns the site element and
+// the thread's first component; consecutive threads take consecutive sites.
+template <int P>
+__device__ __forceinline__ long long split_part(long long e, long long n, int& c0)
+{
+    if constexpr (VecSplit<P>::threads == 1) {
+        c0 = 0;
+        return e;
+    } else {
+        const int q = (e >= n) + (e >= 2 * n) + (e >= 3 * n);
+        c0 = 3 * q;
+        return e - q * n;
+    }
+}
+
 template <int P>
 __global__ void __launch_bounds__(256) update_p_kernel(char* p, const char* r, const char* v,
                                                        Vec2 vec, const Scal* sc)
@@ -110,13 +133,15 @@ __global__ void __launch_bounds__(256) update_p_kernel(char* p, const char* r, c
         for (int k = 0; k < 4; ++k) coef[k] = c[k];
     }
     __syncthreads();
-    const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (j >= vec.nhalf * vec.Vh) return;
+    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x, n = vec.nhalf * vec.Vh;
+    if (e >= VecSplit<P>::threads * n) return;
     long long off;
-    const long long i = split_index(vec, j, off);
+    int c0;
+    const long long i = split_index(vec, split_part<P>(e, n, c0), off);
     off += rhs * vec.rstride;
     const double c[4] = {coef[0], coef[1], coef[2], coef[3]};
-    p_update_site<P>(p + off, r + off, v + off, vec.Vh, i, c, S.fresh != 0);
+    if constexpr (P == WL_F64) p_update_part<3>(p + off, r + off, v + off, vec.Vh, i, c0, c, S.fresh != 0);
+    else p_update_site<P>(p + off, r + off, v + off, vec.Vh, i, c, S.fresh != 0);
 }
 
 template <int P>
@@ -133,12 +158,14 @@ __global__ void __launch_bounds__(256) update_s_kernel(char* s, const char* r, c
         coef[1] = al.im;
     }
     __syncthreads();
-    const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (j >= vec.nhalf * vec.Vh) return;
+    const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x, n = vec.nhalf * vec.Vh;
+    if (e >= VecSplit<P>::threads * n) return;
     long long off;
-    const long long i = split_index(vec, j, off);
+    int c0;
+    const long long i = split_index(vec, split_part<P>(e, n, c0), off);
     off += rhs * vec.rstride;
-    s_update_site<P>(s + off, r + off, v + off, vec.Vh, i, {coef[0], coef[1]});
+    if constexpr (P == WL_F64) s_update_part<3>(s + off, r + off, v + off, vec.Vh, i, c0, {coef[0], coef[1]});
+    else s_update_site<P>(s + off, r + off, v + off, vec.Vh, i, {coef[0], coef[1]});
 }
 
 template <int P, int PX>
@@ -164,13 +191,19 @@ __global__ void __launch_bounds__(256) update_xr_kernel(char* x, Vec2 vx, char* 
     const double dc[4] = {dcoef[0], dcoef[1], dcoef[2], dcoef[3]};
     const bool fresh = S.fresh != 0;
     T tpart[3] = {0, 0, 0};  // this thread's sites in the kernel's arithmetic
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < vec.nhalf * vec.Vh;
-         j += (long long)gridDim.x * blockDim.x) {
+    const long long n = vec.nhalf * vec.Vh;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < VecSplit<P>::threads * n;
+         e += (long long)gridDim.x * blockDim.x) {
         long long off, offx;
-        const long long i = split_index(vec, j, off);
+        int c0;
+        const long long j = split_part<P>(e, n, c0), i = split_index(vec, j, off);
         split_index(vx, j, offx);
         off += rhs * vec.rstride;
         offx += rhs * vx.rstride;
+        if constexpr (P == WL_F64) {
+            xr_update_part<3>(x + offx, r + off, p + off, s + off, t + off, rh + off, vec.Vh, i, c0, dc, tpart, fresh);
+            continue;
+        }
         T pt[3];
         xr_update_site<P, PX>(x + offx, r + off, p + off, s + off, t + off, rh + off, vec.Vh, i,
                               dc, pt, fresh);
@@ -281,6 +314,16 @@ static int ws_alloc(void** p, size_t bytes)
     return WL_OK;
 }
 
+// Threads per block of the per-iteration vector kernels over n elements: 256,
+// or fewer on small lattices, so that the grid still reaches every SM (an 8^4
+// FP64 solve's updates are bound by the FP64 pipes of the SMs they run on).
+static int vec_block(long long n, int sms)
+{
+    int b = kBlock;
+    while (b > 32 && (n + b - 1) / b < 2LL * sms) b >>= 1;
+    return b;
+}
+
 int ensure_ws(wl_gauge g, int inner, int nrhs, int eo)
 {
     Workspace* w = g->ws;
@@ -331,8 +374,10 @@ int ensure_ws(wl_gauge g, int inner, int nrhs, int eo)
     std::memset(w->sc_h, 0, sizeof(Scal) * n);
     // reduction scratch for every kernel the solve launches (no growth later,
     // so graph capture never needs to allocate)
-    const long long hop_blocks = 2 * ((Vh + 31) / 32);  // smallest hop tile: 32 sites
-    const long long blas_blocks = (2 * Vh + kBlock - 1) / kBlock;
+    const long long hop_blocks = 2 * ((Vh + 15) / 16);  // smallest hop tile: 16 sites
+    const long long elements = w->nhalf * Vh * vec_split(inner);  // the updates' (enqueue_iteration)
+    const int vb = vec_block(elements, g->num_sms);
+    const long long blas_blocks = std::max((2 * Vh + kBlock - 1) / kBlock, (elements + vb - 1) / vb);
     WL_TRY(ensure_red(g, nrhs, hop_blocks > blas_blocks ? hop_blocks : blas_blocks));
     return WL_OK;
 }
@@ -415,23 +460,14 @@ static int apply_A(wl_gauge g, Workspace* w, int prec, void* out, const void* in
     return launch_hop(g, h, s);
 }
 
-// Threads per block of the per-iteration vector kernels over n elements: 256,
-// or fewer on small lattices, so that the grid still reaches every SM (an 8^4
-// FP64 solve's updates are bound by the FP64 pipes of the SMs they run on).
-static int vec_block(long long n, int sms)
-{
-    int b = kBlock;
-    while (b > 32 && (n + b - 1) / b < 2LL * sms) b >>= 1;
-    return b;
-}
-
 static int enqueue_iteration(wl_gauge g, Workspace* w, int nrhs, cudaStream_t s)
 {
     const int P = w->inner;
     const Vec2 v = vec_of(g, P, w->nhalf);
     const Vec2 vx = vec_of(g, w->xlo_prec, w->nhalf);
-    const int vb = vec_block(w->nhalf * g->geo.Vh, g->num_sms);
-    const dim3 grid((unsigned)((w->nhalf * g->geo.Vh + vb - 1) / vb), (unsigned)nrhs);
+    const long long elements = w->nhalf * g->geo.Vh * vec_split(P);
+    const int vb = vec_block(elements, g->num_sms);
+    const dim3 grid((unsigned)((elements + vb - 1) / vb), (unsigned)nrhs);
     const int* active = &w->sc[0].active;
     WL_TRY(dispatch_prec(P, [&](auto pc) -> int {
         constexpr int PP = decltype(pc)::value;
@@ -451,12 +487,16 @@ static int enqueue_iteration(wl_gauge g, Workspace* w, int nrhs, cudaStream_t s)
     WL_TRY(apply_A(g, w, P, w->t, w->s, w->s, w->sc[0].st, active, nrhs, s));
     return dispatch_prec(P, [&](auto pc) -> int {
         constexpr int PP = decltype(pc)::value;
-        // grid of resident blocks: the fused reduction leaves few partials
+        // grid of resident blocks: the fused reduction leaves few partials; FP64
+        // blocks of at least 128 threads, whose four warps share the SM's schedulers
+        const int vb = PP == WL_F64 ? std::max(vec_block(elements, g->num_sms), 128) : vec_block(elements, g->num_sms);
         dim3 rgrid = grid;
-        rgrid.x = std::min(grid.x, (unsigned)resident_grid(
+        rgrid.x = (unsigned)((elements + vb - 1) / vb);
+        rgrid.x = std::min(rgrid.x, (unsigned)resident_grid(
                                        w->xlo_prec == WL_F64 ? (const void*)update_xr_kernel<PP, WL_F64>
                                                              : (const void*)update_xr_kernel<PP, WL_F32>,
                                        vb, 0));
+        rgrid.x = std::min(rgrid.x, (unsigned)g->red.max_blocks);  // (ensure_ws made it large enough)
         if (w->xlo_prec == WL_F64)
             update_xr_kernel<PP, WL_F64><<<rgrid, vb, 0, s>>>(
                 (char*)w->xlo, vx, (char*)w->r, (const char*)w->p, (const char*)w->s,
@@ -476,13 +516,12 @@ static int run_chunk_impl(wl_gauge g, Workspace* w, int nrhs, int k, bool use_gr
 
 // Run k iterations and remember what they were charged (see discount_chunk).
 // The autotuner cannot time launches inside a stream capture, so before the
-// first captured chunk for this many right-hand sides v = M p is applied once
-// outside it, which times the iteration's hopping launches.  At a chunk
-// boundary v = M p already holds (p = v = 0 at a round's start), and the
-// per-site results do not depend on the launch shape, so v keeps its value;
-// tmp and the dot product are recomputed before they are read.  The launches
-// are tuning, not solve work: they leave the counters and timing records as
-// they were.  (Eager chunks tune their launches themselves.)
+// first captured chunk for this many right-hand sides v = M r is applied once
+// outside it, which times the iteration's hopping launches.  That chunk is the
+// first of a round, whose first iteration takes p = r and computes v, tmp and the
+// dot product before they are read.  The launches are tuning, not solve work:
+// they leave the counters and timing records as they were.  (Eager chunks tune
+// their launches themselves.)
 static int tune_iteration(wl_gauge g, Workspace* w, int nrhs, bool use_graph, cudaStream_t s)
 {
     if (w->tuned_nrhs == nrhs) return WL_OK;
@@ -490,7 +529,7 @@ static int tune_iteration(wl_gauge g, Workspace* w, int nrhs, bool use_graph, cu
         const long long c0 = g_launches.load(), b0 = g_bytes.load();
         const bool timed = g->timing.on;
         g->timing.on = false;
-        const int rc = apply_A(g, w, w->inner, w->v, w->p, w->rh, w->sc[0].rv, nullptr, nrhs, s);
+        const int rc = apply_A(g, w, w->inner, w->v, w->r, w->rh, w->sc[0].rv, nullptr, nrhs, s);
         g->timing.on = timed;
         g_launches.fetch_sub(g_launches.load() - c0);
         g_bytes.fetch_sub(g_bytes.load() - b0);
@@ -746,7 +785,8 @@ int inner_start(wl_gauge g, Workspace* w, int nrhs, const double* target2,
         auto go = [&](auto* kernel) -> int {
             const int vb = vec_block(w->nhalf * g->geo.Vh, g->num_sms);
             const int resident = (resident_grid((const void*)kernel, vb, 0) + nrhs - 1) / nrhs;
-            const int blocks = (int)std::min<long long>((w->nhalf * g->geo.Vh + vb - 1) / vb, resident);
+            const int blocks = (int)std::min<long long>(std::min<long long>((w->nhalf * g->geo.Vh + vb - 1) / vb, resident),
+                                                        g->red.max_blocks);
             kernel<<<dim3((unsigned)blocks, (unsigned)nrhs), vb, 0, s>>>((char*)w->r, (char*)w->rh, v, (const char*)w->rsrc,
                                                                           vs, w->mask, w->sc, g->red);
             WL_CHECK_LAUNCH((double)(vs.hb + 2 * v.hb) * w->nhalf * nrhs);

@@ -104,7 +104,7 @@ __device__ __forceinline__ void beta_omega(const Scal& S, double (&c)[4])
 {
     const cx<double> rho = {S.rr[0], S.rr[1]}, rp = {S.rho_prev[0], S.rho_prev[1]};
     const cx<double> al = {S.alpha[0], S.alpha[1]}, om = {S.omega[0], S.omega[1]};
-    const cx<double> beta = cdiv(rho, rp) * cdiv(al, om);
+    const cx<double> beta = cdiv(rho * al, rp * om);  // (one complex division: its FP64 chain is every block's start)
     c[0] = beta.re;
     c[1] = beta.im;
     c[2] = om.re;
@@ -209,6 +209,83 @@ __device__ __forceinline__ void xr_update_site(char* x, char* r, const char* p, 
     part[0] = cr;
     part[1] = ci;
     part[2] = nn;
+}
+
+// The three updates on NC FP64 components from c0 on: several threads per site.
+// A warp's FP64 operation takes a scheduler's pipe 64 clocks, so one thread
+// per site leaves a small lattice's updates to a few of them (8^4: update_p
+// 10.1 us, update_s 8.0, update_xr 22.8; with three components per thread
+// 6.6, 5.7 and 12.7).
+template <int NC>
+__device__ __forceinline__ void load_part(cx<double> (&v)[NC], const char* base, long long Vh, long long i, int c0)
+{
+    const double2* p = (const double2*)base + c0 * Vh + i;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const double2 t = p[c * Vh];
+        v[c] = {t.x, t.y};
+    }
+}
+template <int NC>
+__device__ __forceinline__ void store_part(char* base, long long Vh, long long i, int c0, const cx<double> (&v)[NC])
+{
+    double2* p = (double2*)base + c0 * Vh + i;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) p[c * Vh] = make_double2(v[c].re, v[c].im);
+}
+template <int NC>
+__device__ __forceinline__ void p_update_part(char* p, const char* r, const char* v, long long Vh, long long i, int c0,
+                                              const double (&c)[4], bool fresh)
+{
+    cx<double> rr[NC];
+    load_part(rr, r, Vh, i, c0);
+    if (!fresh) {
+        const cx<double> beta = {c[0], c[1]}, om = {c[2], c[3]};
+        cx<double> pp[NC], vv[NC];
+        load_part(pp, p, Vh, i, c0);
+        load_part(vv, v, Vh, i, c0);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) rr[k] = rr[k] + beta * (pp[k] - om * vv[k]);
+    }
+    store_part(p, Vh, i, c0, rr);
+}
+template <int NC>
+__device__ __forceinline__ void s_update_part(char* s, const char* r, const char* v, long long Vh, long long i, int c0,
+                                              cx<double> al)
+{
+    cx<double> rr[NC], vv[NC];
+    load_part(rr, r, Vh, i, c0);
+    load_part(vv, v, Vh, i, c0);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) rr[k] = rr[k] - al * vv[k];
+    store_part(s, Vh, i, c0, rr);
+}
+template <int NC>
+__device__ __forceinline__ void xr_update_part(char* x, char* r, const char* p, const char* s, const char* t, const char* rh,
+                                               long long Vh, long long i, int c0, const double (&dc)[4], double (&part)[3],
+                                               bool fresh)
+{
+    const cx<double> al = {dc[0], dc[1]}, om = {dc[2], dc[3]};
+    cx<double> pp[NC], ss[NC], xx[NC], tt[NC], hh[NC];
+    load_part(pp, p, Vh, i, c0);
+    load_part(ss, s, Vh, i, c0);
+    load_part(tt, t, Vh, i, c0);
+    load_part(hh, rh, Vh, i, c0);
+    if (!fresh) load_part(xx, x, Vh, i, c0);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const cx<double> d = al * pp[k] + om * ss[k];
+        xx[k] = fresh ? d : xx[k] + d;
+    }
+    store_part(x, Vh, i, c0, xx);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        ss[k] = ss[k] - om * tt[k];
+        part[0] = fma(hh[k].re, ss[k].re, fma(hh[k].im, ss[k].im, part[0]));
+        part[1] = fma(hh[k].re, ss[k].im, fma(-hh[k].im, ss[k].re, part[1]));
+        part[2] = fma(ss[k].re, ss[k].re, fma(ss[k].im, ss[k].im, part[2]));
+    }
+    store_part(r, Vh, i, c0, ss);
 }
 
 // The last block of the x/r update advances one right-hand side's scalars and
