@@ -203,9 +203,11 @@ static int tuned_shape(wl_gauge g, const HopLaunch& h, int lf, HopArgs& A, int n
 {
     const bool multi = nrhs > 1;
     const int dflt = multi ? (nrhs < 8 ? nrhs : 8) : kHopBlock;
-    char key[96];
-    snprintf(key, sizeof key, "hop p%d d%d dot%d np%d r%d x%d%d w%d c%d l%d", h.prec, h.dagger, (int)h.dot,
-             h.nparity, nrhs, h.x1[0] != nullptr, h.x2[0] != nullptr, h.w[0] != nullptr, h.cl_mode, lf);
+    // one bit field per property of the launch (nrhs is at most kMaxRhsLaunch)
+    const int field[][2] = {{h.prec, 2}, {h.dagger, 1}, {(int)h.dot, 1}, {h.nparity, 2}, {nrhs, 6}, {h.x1[0] != nullptr, 1},
+                            {h.x2[0] != nullptr, 1}, {h.w[0] != nullptr, 1}, {h.cl_mode, 2}, {lf, 2}};
+    unsigned long long key = 0;
+    for (const auto& f : field) key = key << f[1] | (unsigned)f[0];
     auto it = g->tuned.find(key);
     if (it != g->tuned.end()) {
         *shape = it->second.block;
@@ -295,7 +297,8 @@ static int tuned_shape(wl_gauge g, const HopLaunch& h, int lf, HopArgs& A, int n
         if (best_t[ci] < best_t[bi]) bi = ci;
     const int best_shape = cand[bi];
     if (getenv("WL_AUTOTUNE_VERBOSE")) {
-        fprintf(stderr, "[wl autotune] %s Vh=%lld:", key, g->geo.Vh);
+        fprintf(stderr, "[wl autotune] hop p%d d%d dot%d np%d r%d x%d%d w%d c%d l%d Vh=%lld:", h.prec, h.dagger, (int)h.dot,
+                h.nparity, nrhs, h.x1[0] != nullptr, h.x2[0] != nullptr, h.w[0] != nullptr, h.cl_mode, lf, g->geo.Vh);
         for (size_t ci = 0; ci < cand.size(); ++ci) fprintf(stderr, " %d:%.1fus", cand[ci], best_t[ci] * 1e3f);
         fprintf(stderr, " -> %d\n", best_shape);
     }

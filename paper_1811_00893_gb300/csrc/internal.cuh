@@ -5,6 +5,7 @@
 #include <map>
 #include <memory>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "common.cuh"
@@ -77,7 +78,7 @@ struct wl_gauge_s {
     // clover term (clover.cu): [prec][parity][0: A = 1 + F, 1: A^-1]
     void* clov[4][2][2] = {};
     bool has_clover = false;
-    std::map<std::string, wl::Tuned> tuned;
+    std::unordered_map<unsigned long long, wl::Tuned> tuned;  // key: dslash.cu tuned_shape
     // set for a block of a domain decomposition (wl_dd): its links see the
     // neighbouring blocks across the cut faces, so only the _dd calls apply it
     int dd_part = 0;

@@ -61,6 +61,8 @@ class wl_solve_info(ctypes.Structure):
                 ("secs", ctypes.c_double)]
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda device: torch.cuda.current_stream(device).cuda_stream)
 _lock = threading.Lock()
 _lib = None
 LIB_PATH = _build.LIB
@@ -160,7 +162,9 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # torch.cuda.current_stream() builds a Stream object (2.9 us of an 8 us
+        # wilson_dslash call on the host cores of a GB300); this is its handle alone
+        return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
     if isinstance(stream, torch.cuda.Stream):
         return ctypes.c_void_p(stream.cuda_stream)
     return ctypes.c_void_p(int(stream))
