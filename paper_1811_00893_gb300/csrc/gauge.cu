@@ -338,14 +338,26 @@ __global__ void build_links_r8_kernel(void* out, const double* __restrict__ U, G
 // to the other parity, and an internal field has one plane per component (pair):
 // one thread per site on the canonical side would touch 32 sites' 192-byte
 // runs with each warp access.  A block moves kConvSites sites through shared
-// memory instead: 12 consecutive threads move one site's 12 complex numbers on the
-// canonical side, one thread per site its planes on the internal side.  HBM
-// bound, on runs of 192 bytes every 384: FP32, 24^3 x 48, 12 right-hand sides
-// (1.15 GB either way, 169 us at the copy rate): to canonical 666 us with one
-// thread per site, 212 us so; to
-// internal 264 us, 259 us (288 us without cp.async).  The FP64 <-> FP32 conversions run on the integer pipes (df64.cuh).
-static constexpr int kConvSites = 128;
-static constexpr int kConvPitch = kConvSites + 1;  // 16-byte words: neighbouring components in different banks
+// memory instead, one bulk copy of 192 bytes per site on the canonical side and
+// one thread per site on the internal side.  HBM bound, on runs of 192 bytes
+// every 384: a bulk copy fetches those bytes, while loads (and cp.async) fetch
+// whole 128-byte lines, a third more than is used.  FP32, 24^3 x 48, 12
+// right-hand sides (1.15 GB either way, 169 us at the copy rate): to internal
+// 264 us with one thread per site, 262 us by cp.async, 235 us by 32-byte loads,
+// 203 us by bulk copies; to canonical 666, 223 (16- or 32-byte stores) and
+// 205 us.  The FP64 <-> FP32 conversions run on the integer pipes (df64.cuh).
+static constexpr int kConvSites = 64;
+static constexpr int kConvPitch = 13;  // 16-byte words per site: neighbouring sites in different banks
+
+// Wait for phase 0 of an mbarrier; false if it did not complete (after seconds).
+__device__ __forceinline__ bool bulk_wait(unsigned bar)
+{
+    unsigned done = 0;
+    for (int k = 0; k < (1 << 22) && !done; ++k)
+        asm volatile("{\n .reg .pred q;\n mbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\n selp.u32 %0, 1, 0, q;\n}"
+                     : "=r"(done) : "r"(bar) : "memory");
+    return done != 0;
+}
 
 // canonical index of half site i of parity p, by the fast divisions (below 2^31)
 __device__ __forceinline__ long long canonical_site(const Geom& g, int p, int i)
@@ -362,73 +374,65 @@ template <int P>
 __global__ void __launch_bounds__(kConvSites) to_internal_kernel(char* out, const double* __restrict__ in, Geom g, int p,
                                                                  size_t fb, long long V)
 {
-    __shared__ double2 sm[12 * kConvPitch];
-    __shared__ unsigned where[kConvSites];
-    const int rhs = blockIdx.y, base = blockIdx.x * kConvSites;
+    __shared__ __align__(16) double2 sm[kConvSites * kConvPitch];
+    __shared__ __align__(8) unsigned long long landed;
+    const int rhs = blockIdx.y, base = blockIdx.x * kConvSites, j = threadIdx.x;
     const int n = (int)min((long long)kConvSites, g.Vh - base);
-    if ((int)threadIdx.x < n) where[threadIdx.x] = (unsigned)canonical_site(g, p, base + threadIdx.x);
-    __syncthreads();
-    if (((size_t)in & 15) == 0) {  // cp.async: every copy of the block in flight, no register waits
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const int e = k * kConvSites + threadIdx.x, j = e / 12, c = e - 12 * j;
-            if (j < n) cp_async16(sm + c * kConvPitch + j, in + (((long long)rhs * V + where[j]) * 12 + c) * 2);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-    } else {  // callers' fields are aligned to 8 bytes at least
-        for (int k = 0; k < 12; ++k) {
-            const int e = k * kConvSites + threadIdx.x, j = e / 12, c = e - 12 * j;
-            if (j >= n) break;
-            const double* q = in + (((long long)rhs * V + where[j]) * 12 + c) * 2;
-            sm[c * kConvPitch + j] = make_double2(__ldg(q), __ldg(q + 1));
-        }
+    const bool bulk = ((size_t)in & 15) == 0;  // callers' fields are aligned to 8 bytes at least
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(&landed);
+    if (bulk && j == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(192 * n) : "memory");
     }
     __syncthreads();
-    if ((int)threadIdx.x >= n) return;
+    if (j >= n) return;
+    const double* site = in + ((long long)rhs * V + canonical_site(g, p, base + j)) * 24;
+    double2* u = sm + j * kConvPitch;
+    bool ok = true;
+    if (bulk) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], 192, [%2];" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(u)),
+                     "l"(site), "r"(bar)
+                     : "memory");
+        ok = bulk_wait(bar);
+    } else {
+        for (int c = 0; c < 12; ++c) u[c] = make_double2(__ldg(site + 2 * c), __ldg(site + 2 * c + 1));
+    }
     using T = typename Prec<P>::real;
     cx<T> v[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-        const double2 u = sm[c * kConvPitch + threadIdx.x];
-        v[c] = {cast<T>(u.x), cast<T>(u.y)};
+        v[c] = {cast<T>(u[c].x), cast<T>(u[c].y)};
+        if (!ok) v[c] = {cast<T>(nan("")), cast<T>(nan(""))};  // (a copy that never landed shows)
     }
-    store_spinor<P>(out + rhs * fb, g.Vh, base + threadIdx.x, v);
+    store_spinor<P>(out + rhs * fb, g.Vh, base + j, v);
 }
 
-// (the narrow types pass through shared memory in FP32: half the space, twice the resident blocks)
 template <int P>
 __global__ void __launch_bounds__(kConvSites) to_canonical_kernel(double* out, const char* in, Geom g, int p, size_t fb,
                                                                   long long V)
 {
-    constexpr bool narrow = P == WL_F32 || P == WL_F16;
-    using W = typename std::conditional<narrow, float2, double2>::type;
-    using S = typename std::conditional<narrow, float, double>::type;
-    __shared__ W sm[12 * kConvPitch];
-    __shared__ unsigned where[kConvSites];
-    const int rhs = blockIdx.y, base = blockIdx.x * kConvSites;
-    const int n = (int)min((long long)kConvSites, g.Vh - base);
-    if ((int)threadIdx.x < n) {
-        cx<typename Prec<P>::real> v[12];
-        load_spinor<P>(v, in + rhs * fb, g.Vh, base + threadIdx.x);
-        where[threadIdx.x] = (unsigned)canonical_site(g, p, base + threadIdx.x);
+    __shared__ __align__(16) double2 sm[kConvSites * kConvPitch];
+    const int rhs = blockIdx.y, base = blockIdx.x * kConvSites, j = threadIdx.x;
+    if (j >= (int)min((long long)kConvSites, g.Vh - base)) return;
+    cx<typename Prec<P>::real> v[12];
+    load_spinor<P>(v, in + rhs * fb, g.Vh, base + j);
+    double* site = out + ((long long)rhs * V + canonical_site(g, p, base + j)) * 24;
+    double2* u = sm + j * kConvPitch;
 #pragma unroll
-        for (int c = 0; c < 12; ++c) sm[c * kConvPitch + threadIdx.x] = {cast<S>(v[c].re), cast<S>(v[c].im)};
-    }
-    __syncthreads();
-    const bool wide = ((size_t)out & 15) == 0;  // callers' fields are aligned to 8 bytes at least
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const int e = k * kConvSites + threadIdx.x, j = e / 12, c = e - 12 * j;
-        if (j >= n) continue;
-        double* q = out + (((long long)rhs * V + where[j]) * 12 + c) * 2;
-        const W u = sm[c * kConvPitch + j];
-        const double2 d = make_double2(cast<double>(u.x), cast<double>(u.y));
-        if (wide) {
-            *(double2*)q = d;
-        } else {
-            q[0] = d.x;
-            q[1] = d.y;
+    for (int c = 0; c < 12; ++c) u[c] = make_double2(cast<double>(v[c].re), cast<double>(v[c].im));
+    if (((size_t)out & 15) == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 192;" ::"l"(site),
+                     "r"((unsigned)__cvta_generic_to_shared(u))
+                     : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    } else {  // callers' fields are aligned to 8 bytes at least
+        for (int c = 0; c < 12; ++c) {
+            site[2 * c] = u[c].x;
+            site[2 * c + 1] = u[c].y;
         }
     }
 }
