@@ -108,12 +108,14 @@ __global__ void __launch_bounds__(256) cdot_kernel(const void* a, const void* b,
                 }
                 nn = fma(y[u][c].re, y[u][c].re, fma(y[u][c].im, y[u][c].im, nn));
             }
-            if constexpr (NORM) cr = nn;
-            part[0] += (double)cr;
-            part[1] += (double)ci;
+            if constexpr (!NORM) {
+                part[0] += (double)cr;
+                part[1] += (double)ci;
+            }
             part[2] += (double)nn;
         }
     }
+    if constexpr (NORM) part[0] = part[2];
     __shared__ double sh[3 * 32];
     block_sum<3>(part, sh);
     double tot[3];
@@ -213,9 +215,12 @@ int launch_cdot(wl_gauge g, int prec, const void* a, const void* b, int nhalf, i
                        : prec == WL_F32 ? (const void*)cdot_kernel<WL_F32, false>
                        : prec == WL_F16 ? (const void*)cdot_kernel<WL_F16, false>
                                         : (const void*)cdot_kernel<WL_DF64, false>;
-    // resident blocks in all: the FP64 sums over a block's threads cost more
-    // than a few sites' loads
-    grid.x = std::min(grid.x, (unsigned)((resident_grid(kern, kBlasBlock, 0) + nrhs - 1) / nrhs));
+    // Resident blocks in all: the FP64 sums over a block's threads cost more
+    // than a few sites' loads.  Rounded down: a few blocks more than fit are a
+    // second wave (24^3 x 48, 12 right-hand sides, 612 blocks or 600 on 608
+    // places: FP32 146 and 112 us, its norm 78 and 60, FP16 103 and 70, FP64
+    // 716 and 504).
+    grid.x = std::min(grid.x, (unsigned)std::max(resident_grid(kern, kBlasBlock, 0) / nrhs, 1));
     WL_TRY(ensure_red(g, nrhs, grid.x));
     const Vec v = make_vec(g, prec, nhalf, rs);
     auto go = [&](auto nt) {

@@ -784,7 +784,7 @@ int inner_start(wl_gauge g, Workspace* w, int nrhs, const double* target2,
         constexpr int PP = decltype(pc)::value;
         auto go = [&](auto* kernel) -> int {
             const int vb = vec_block(w->nhalf * g->geo.Vh, g->num_sms);
-            const int resident = (resident_grid((const void*)kernel, vb, 0) + nrhs - 1) / nrhs;
+            const int resident = std::max(resident_grid((const void*)kernel, vb, 0) / nrhs, 1);  // (one wave)
             const int blocks = (int)std::min<long long>(std::min<long long>((w->nhalf * g->geo.Vh + vb - 1) / vb, resident),
                                                         g->red.max_blocks);
             kernel<<<dim3((unsigned)blocks, (unsigned)nrhs), vb, 0, s>>>((char*)w->r, (char*)w->rh, v, (const char*)w->rsrc,
