@@ -499,6 +499,27 @@ __device__ __forceinline__ void warp_sum<3, double>(double (&v)[3])
     warp_sum3(v);
 }
 
+// Sum of the block's per-warp totals in sh (warp 0).  Up to eight warps: one
+// lane per component adds them one by one, nw - 1 dependent additions of one
+// warp instruction each, where warp_sum takes 7.
+template <int N>
+__device__ __forceinline__ void sum_warp_totals(double (&v)[N], const double* sh, int lane, int nw)
+{
+    if (nw <= 8) {
+        double t = 0.0;
+        if (lane < N) {
+            t = sh[lane * 32];
+            for (int k = 1; k < nw; ++k) t += sh[lane * 32 + k];
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = __shfl_sync(0xffffffffu, t, k);
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = lane < nw ? sh[k * 32 + lane] : 0.0;
+    warp_sum<N>(v);
+}
+
 // Sum v over the block; the total is valid in thread 0.  `sh` holds
 // N * 32 doubles.
 template <int N>
@@ -511,11 +532,7 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* sh)
 #pragma unroll
         for (int k = 0; k < N; ++k) sh[k * 32 + w] = v[k];
     __syncthreads();
-    if (w == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) v[k] = lane < nw ? sh[k * 32 + lane] : 0.0;
-        warp_sum<N>(v);
-    }
+    if (w == 0) sum_warp_totals<N>(v, sh, lane, nw);
 }
 
 // Block sum of per-warp totals already formed in a narrower type: lane 0 of
@@ -531,11 +548,7 @@ __device__ __forceinline__ void block_sum_warps(double (&v)[N], double* sh)
 #pragma unroll
         for (int k = 0; k < N; ++k) sh[k * 32 + w] = v[k];
     __syncthreads();
-    if (w == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) v[k] = lane < nw ? sh[k * 32 + lane] : 0.0;
-        warp_sum<N>(v);
-    }
+    if (w == 0) sum_warp_totals<N>(v, sh, lane, nw);
 }
 
 // This thread's share of the sum of nblocks partial N-tuples (stride N),

@@ -348,10 +348,11 @@ __global__ void __launch_bounds__(kFxRowBlock) hop_fx_rows_kernel(const HopArgs 
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
                 const long long o = (3 * (j + 2 * s) + a) * Vh + i;
-                if (A.a != 1.0) v[s] = A.a * v[s];
                 if (x1) {
                     const double2 t = x1[o];
-                    v[s] = v[s] + cx<double>{t.x, t.y};
+                    v[s] = {fma(A.a, v[s].re, t.x), fma(A.a, v[s].im, t.y)};
+                } else if (A.a != 1.0) {
+                    v[s] = A.a * v[s];
                 }
                 if (x2) {
                     const double2 t = x2[o];
@@ -446,13 +447,14 @@ __global__ void __launch_bounds__(3 * kRowSites) hop_rows_kernel(const HopArgs A
         const double sa = A.a, b1 = A.b1;
         cx<double> v[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) v[s] = sa == 1.0 ? acc[3 * s] : sa * acc[3 * s];
-        if (x1)
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
+        for (int s = 0; s < 4; ++s) {
+            if (x1) {
                 const double2 t = x1[(3 * s + a) * Vh + i];
-                v[s] = v[s] + cx<double>{t.x, t.y};
+                v[s] = {fma(sa, acc[3 * s].re, t.x), fma(sa, acc[3 * s].im, t.y)};
+            } else {
+                v[s] = sa == 1.0 ? acc[3 * s] : sa * acc[3 * s];
             }
+        }
         if (x2)
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
