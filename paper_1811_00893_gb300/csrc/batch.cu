@@ -137,6 +137,10 @@ __global__ void __launch_bounds__(256) batch_hop_kernel(const BatchArgs B)
                     w = L.s + o;
                     a = -L.kappa2;
                 }
+                if (DOT && kPrefetchMulti<P>) {
+                    prefetch_spinor_l2<P>(x1, L.g.Vh, i);
+                    if (w != x1) prefetch_spinor_l2<P>(w, L.g.Vh, i);
+                }
                 cx<T> acc[12];
                 if constexpr (P == WL_F64) {
                     if (L.fx64) hop_site<P, false, 3>(acc, nb, L.g.Vh, in, smem, kTile, lane);

@@ -936,6 +936,32 @@ __device__ __forceinline__ void epilogue_ptrs(cx<typename Prec<P>::real> (&acc)[
     }
 }
 
+// Ask L2 for the site's epilogue operands (x1, x2, w) before the stencil
+// starts, so that their loads after the eight hops do not wait on HBM.  A
+// prefetch holds no register.  One right-hand side: FP16 solve 149.8 -> 148.5
+// ms, but the FP32 hop 141 -> 151 us (its register budget tips into spills), so
+// only FP16 prefetches; fixed-point FP64 (bound by integer issue) 71.3 -> 73.7
+// us for D of 20x18x14x30.  Links shared by several right-hand sides: D-hat of
+// 24^3 x 48 in FP32 with 12 of them 549 -> 535 us.
+// WL_PREFETCH_EPILOGUE=0 builds without it.
+#ifndef WL_PREFETCH_EPILOGUE
+#define WL_PREFETCH_EPILOGUE 1
+#endif
+template <int P>
+static constexpr bool kPrefetchSingle = WL_PREFETCH_EPILOGUE && P == WL_F16;
+template <int P>
+static constexpr bool kPrefetchMulti = WL_PREFETCH_EPILOGUE && (P == WL_F16 || P == WL_F32);
+
+template <int P>
+__device__ __forceinline__ void prefetch_spinor_l2(const char* base, long long Vh, long long i)
+{
+    constexpr int planes = (P == WL_F32) ? 6 : (P == WL_F16) ? 3 : 12;  // 16-byte planes
+#pragma unroll
+    for (int k = 0; k < planes; ++k)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (k * Vh + i) * 16));
+    if (P == WL_F16) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + 3 * Vh * 16 + i * 4));
+}
+
 template <int P, bool DOT, int CL = kClNone>
 __device__ __forceinline__ void epilogue(cx<typename Prec<P>::real> (&acc)[12], const HopArgs& A,
                                          int pidx, int rhs, int i, typename Prec<P>::real (&part)[3])

@@ -48,22 +48,13 @@ struct MinBlocks {
     static constexpr int value = DOT && base > 2 ? 2 : base;  // the reducing loop needs more
 };
 
-// Ask L2 for the site's epilogue operands (x1, x2, w) before the stencil
-// starts, so that their loads after the eight hops do not wait on HBM.  A
-// prefetch holds no register.  Measured: FP16 solve 149.8 -> 148.5 ms, but
-// the FP32 hop 141 -> 151 us (its register budget tips into spills), so only
-// the FP16 kernels prefetch.  WL_PREFETCH_EPILOGUE=0 builds without it.
-#ifndef WL_PREFETCH_EPILOGUE
-#define WL_PREFETCH_EPILOGUE 1
-#endif
-template <int P>
-__device__ __forceinline__ void prefetch_spinor_l2(const char* base, long long Vh, long long i)
+template <int P, bool DOT>
+__device__ __forceinline__ void prefetch_epilogue(const HopArgs& A, int rhs, int pidx, int i)
 {
-    constexpr int planes = (P == WL_F32) ? 6 : (P == WL_F16) ? 3 : 12;  // 16-byte planes
-#pragma unroll
-    for (int k = 0; k < planes; ++k)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (k * Vh + i) * 16));
-    if (P == WL_F16) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + 3 * Vh * 16 + i * 4));
+    if (A.x1[pidx]) prefetch_spinor_l2<P>(A.x1[pidx] + rhs * A.rs_x1, A.g.Vh, i);
+    if (A.x2[pidx]) prefetch_spinor_l2<P>(A.x2[pidx] + rhs * A.rs_x2, A.g.Vh, i);
+    if (DOT && A.w[pidx] && A.w[pidx] != A.x1[pidx])
+        prefetch_spinor_l2<P>(A.w[pidx] + rhs * A.rs_w, A.g.Vh, i);
 }
 
 template <int P, bool DAG, bool DOT, int CL, int LF>
@@ -71,12 +62,7 @@ __device__ __forceinline__ void hop_kernel_site(const HopArgs& A, int rhs, int p
                                                 typename Prec<P>::real (&part)[3])
 {
     using T = typename Prec<P>::real;
-    if (WL_PREFETCH_EPILOGUE && P == WL_F16) {
-        if (A.x1[pidx]) prefetch_spinor_l2<P>(A.x1[pidx] + rhs * A.rs_x1, A.g.Vh, i);
-        if (A.x2[pidx]) prefetch_spinor_l2<P>(A.x2[pidx] + rhs * A.rs_x2, A.g.Vh, i);
-        if (DOT && A.w[pidx] && A.w[pidx] != A.x1[pidx])
-            prefetch_spinor_l2<P>(A.w[pidx] + rhs * A.rs_w, A.g.Vh, i);
-    }
+    if (kPrefetchSingle<P>) prefetch_epilogue<P, DOT>(A, rhs, pidx, i);
     cx<T> acc[12];
     int nb[8];
     unsigned cross = 0;
@@ -157,6 +143,7 @@ __global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_mrhs_
         const bool act = !A.active || A.active[r * A.active_stride] != 0;  // warp-uniform
         T part[3] = {0, 0, 0};
         if (act && valid) {
+            if (kPrefetchMulti<P>) prefetch_epilogue<P, DOT>(A, r, pidx, i);
             cx<T> acc[12];
             hop_site<P, DAG, LF>(acc, nb, A.g.Vh, A.in[pidx] + r * A.rs_in, smem, kTile, lane, cross, A.ph);
             epilogue<P, DOT, CL>(acc, A, pidx, r, i, part);
@@ -237,6 +224,7 @@ __global__ void __launch_bounds__(256, 2) hop_mrhs_pipe_kernel(const HopArgs A, 
             const bool act = !A.active || A.active[r * A.active_stride] != 0;  // warp-uniform
             T part[3] = {0, 0, 0};
             if (act && valid) {
+                if (kPrefetchMulti<P>) prefetch_epilogue<P, DOT>(A, r, pidx, i);
                 cx<T> acc[12];
                 hop_site<P, DAG, LF>(acc, nb, A.g.Vh, A.in[pidx] + r * A.rs_in, links, kTile, lane, cross,
                                      A.ph);
