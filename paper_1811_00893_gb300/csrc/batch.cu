@@ -103,12 +103,19 @@ __global__ void __launch_bounds__(256) batch_hop_kernel(const BatchArgs B)
         const BLat& L = B.lats[s_lat];
         const int base = (item - L.item0) * kTile;
         const int n = (int)min((long long)kTile, L.g.Vh - base);
-        stage_links<P>(smem, (const char*)L.links[par], L.g.Vh, base, n);
-        __syncthreads();
+        stage_links_async<P>(smem, (const char*)L.links[par], L.g.Vh, base, n);
+        cp_async_commit();
         const int i = base + lane;
         const bool valid = lane < n;
+        const char* src = OP == 0 ? L.p : OP == 2 ? L.s : L.tmp;
         int nb[8];
-        if (valid) neighbours(L.g, par, i, nb);
+        if (valid) {
+            neighbours(L.g, par, i, nb);
+            if (kPrefetchMulti<P> && threadIdx.y < L.nrhs)
+                prefetch_spinor_l2<P>(src + threadIdx.y * L.vb, L.g.Vh, nb[6]);
+        }
+        cp_async_wait<0>();
+        __syncthreads();
         for (int r = threadIdx.y; r < L.nrhs; r += blockDim.y) {
             const bool act = L.sc[r].active != 0;  // warp-uniform
             T part[3] = {0, 0, 0};
@@ -137,6 +144,8 @@ __global__ void __launch_bounds__(256) batch_hop_kernel(const BatchArgs B)
                     w = L.s + o;
                     a = -L.kappa2;
                 }
+                if (kPrefetchMulti<P> && r + blockDim.y < L.nrhs)
+                    prefetch_spinor_l2<P>(src + (r + blockDim.y) * L.vb, L.g.Vh, nb[6]);
                 if (DOT && kPrefetchMulti<P>) {
                     prefetch_spinor_l2<P>(x1, L.g.Vh, i);
                     if (w != x1) prefetch_spinor_l2<P>(w, L.g.Vh, i);

@@ -128,9 +128,9 @@ __global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_mrhs_
     const int p = A.parity0 + pidx;
     const int base = (blockIdx.x - pidx * A.blocks_per_parity) * kTile;
     const int n = (int)min((long long)kTile, A.g.Vh - base);
-    stage_links<P, LF>(smem, (const char*)A.links[pidx], A.g.Vh, base, n);
+    stage_links_async<P, LF>(smem, (const char*)A.links[pidx], A.g.Vh, base, n);
+    cp_async_commit();
     double* bpart = (double*)(smem + LinkLayout<P, LF>::bytes * kTile);
-    __syncthreads();
     const int lane = threadIdx.x, i = base + lane;
     const bool valid = lane < n;
     int nb[8];
@@ -138,12 +138,18 @@ __global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_mrhs_
     if (valid) {
         if constexpr (LF == 1 || LF == 2) neighbours(A.g, p, i, nb, cross);
         else neighbours(A.g, p, i, nb);
+        if (kPrefetchMulti<P> && threadIdx.y < nrhs)
+            prefetch_spinor_l2<P>(A.in[pidx] + threadIdx.y * A.rs_in, A.g.Vh, nb[6]);
     }
+    cp_async_wait<0>();
+    __syncthreads();
     for (int r = threadIdx.y; r < nrhs; r += blockDim.y) {
         const bool act = !A.active || A.active[r * A.active_stride] != 0;  // warp-uniform
         T part[3] = {0, 0, 0};
         if (act && valid) {
             if (kPrefetchMulti<P>) prefetch_epilogue<P, DOT>(A, r, pidx, i);
+            if (kPrefetchMulti<P> && r + blockDim.y < nrhs)
+                prefetch_spinor_l2<P>(A.in[pidx] + (r + blockDim.y) * A.rs_in, A.g.Vh, nb[6]);
             cx<T> acc[12];
             hop_site<P, DAG, LF>(acc, nb, A.g.Vh, A.in[pidx] + r * A.rs_in, smem, kTile, lane, cross, A.ph);
             epilogue<P, DOT, CL>(acc, A, pidx, r, i, part);
@@ -225,6 +231,8 @@ __global__ void __launch_bounds__(256, 2) hop_mrhs_pipe_kernel(const HopArgs A, 
             T part[3] = {0, 0, 0};
             if (act && valid) {
                 if (kPrefetchMulti<P>) prefetch_epilogue<P, DOT>(A, r, pidx, i);
+                if (kPrefetchMulti<P> && r + blockDim.y < nrhs)
+                    prefetch_spinor_l2<P>(A.in[pidx] + (r + blockDim.y) * A.rs_in, A.g.Vh, nb[6]);
                 cx<T> acc[12];
                 hop_site<P, DAG, LF>(acc, nb, A.g.Vh, A.in[pidx] + r * A.rs_in, links, kTile, lane, cross,
                                      A.ph);
