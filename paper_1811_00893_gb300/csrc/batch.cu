@@ -70,28 +70,34 @@ __global__ void __launch_bounds__(256) batch_hop_kernel(const BatchArgs B)
     __shared__ bool last;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
     const int lane = threadIdx.x;
+    // Warp 0 takes an item from the counter one item ahead of its use, so that
+    // the counter's latency passes while the block computes, and looks its
+    // lattice up with one load per lane: its last lattice that does not start
+    // after the item, and whether one of that lattice's right-hand sides is
+    // active.  A lattice whose systems are all inactive (converged, or between
+    // rounds) needs neither its links nor any arithmetic.
+    unsigned next = 0;
+    if (tid == 0) next = atomicAdd(&B.queue[0], 1u);
     for (;;) {
-        if (tid == 0) {
-            const int it = (int)atomicAdd(&B.queue[0], 1u);
-            int lo = 0, hi = B.nlat - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (B.lats[mid].item0 <= it) lo = mid;
-                else hi = mid - 1;
-            }
-            s_item = it;
-            s_lat = lo;
-            // a lattice whose systems are all inactive (converged, or between
-            // rounds) needs neither its links nor any arithmetic
+        if (threadIdx.y == 0) {
+            const int it = (int)__shfl_sync(0xffffffffu, next, 0);
+            int lo = -1;
+            for (int l = lane; l < kMaxBatchLat; l += 32)
+                lo += __popc(__ballot_sync(0xffffffffu, l < B.nlat && B.lats[l].item0 <= it));
             int any = 0;
             if (it < B.total_items) {
                 const BLat& Lq = B.lats[lo];
-                for (int r = 0; r < Lq.nrhs && !any; ++r) any = Lq.sc[r].active != 0;
+                any = __any_sync(0xffffffffu, lane < Lq.nrhs && Lq.sc[lane].active != 0);
                 // move the counter past the rest of an idle lattice's items at
                 // once (every item in between belongs to it)
-                if (!any) atomicMax(&B.queue[0], (unsigned)(Lq.item0 + Lq.nitems));
+                if (!any && lane == 0) atomicMax(&B.queue[0], (unsigned)(Lq.item0 + Lq.nitems));
             }
-            s_any = any;
+            if (lane == 0) {
+                s_item = it;
+                s_lat = lo;
+                s_any = any;
+                if (it < B.total_items) next = atomicAdd(&B.queue[0], 1u);
+            }
         }
         __syncthreads();
         const int item = s_item;
