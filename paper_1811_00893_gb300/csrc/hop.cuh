@@ -882,8 +882,9 @@ __device__ __forceinline__ void epilogue_ptrs(cx<typename Prec<P>::real> (&acc)[
     using T = typename Prec<P>::real;
     const T a = (T)a_;
     // FP32 and FP64: one operation for a acc + x1 (FP64: 24 multiplications would
-    // take a tenth of the hop's time)
-    constexpr bool fold = P == WL_F64 || P == WL_F32;
+    // take a tenth of the hop's time; the clover forms, whose x1 is absent in the
+    // iterations, are 0.6 % faster without the choice)
+    constexpr bool fold = CL == kClNone && (P == WL_F64 || P == WL_F32);
     if (!(fold && x1) && (P != WL_F64 || a_ != 1.0))
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = a * acc[c];

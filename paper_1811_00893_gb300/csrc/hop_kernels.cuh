@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(256, 2) hop_mrhs_pipe_kernel(const HopArgs A, 
 // nothing from sharing the links: a form with the links of a tile staged for
 // all of them took 1,727 us for the hopping term of 24^3 x 48 with 12
 // right-hand sides, one grid row per right-hand side 1,434 us.  32^3 x 64,
-// one right-hand side: 390 us, in FP64 arithmetic 1,628 us.  Reducing
+// one right-hand side: 385 us, in FP64 arithmetic 1,628 us.  Reducing
 // launches use the full grid too; the partial sums are added by the last
 // block or (partials_only) by a finishing launch.
 static constexpr int kFxBlock = 64;
