@@ -1,4 +1,4 @@
-"""Layout conversion at the edges of its blocks (128 half sites), for canonical fields
+"""Layout conversion at the edges of its blocks (64 half sites), for canonical fields
 aligned to 16 and to 8 bytes, and the FP64 -> FP32 rounding against IEEE 754's."""
 import numpy as np
 import pytest
