@@ -1,0 +1,121 @@
+"""FP64 hopping term with fixed-point links against exact arithmetic.
+
+The reference is the hopping term in whole numbers: links and spinors are binary64, so
+multiplied by a power of two they are integers, and sums of products of integers have no
+rounding.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1811_00893_gb300 import fields, wilson
+
+pytestmark = pytest.mark.gpu
+
+BC = (1, 1, 1, -1)
+SHAPES = [64, 2000]  # one thread per site; six threads per site
+DIMS = [(2, 2, 2, 2), (6, 2, 2, 2), (4, 4, 4, 4)]  # Vh = 8, 24 (half a tile of 16 sites, one and a half) and 128
+
+
+def _ints(a, bits):
+    """Real and imaginary parts of a complex array times 2^bits, as Python integers."""
+    def conv(r):
+        m, e = np.frexp(np.ascontiguousarray(r))
+        n = np.ldexp(m, 53).astype(np.int64).astype(object)
+        sh = e.astype(np.int64) - 53 + bits
+        assert np.all((sh >= 0) | (r == 0)), "not a multiple of 2^-bits"
+        return n * (2 ** np.maximum(sh, 0).astype(object))
+    return conv(a.real), conv(a.imag)
+
+
+class Exact:
+    """The hopping term of one field in integers: out = (re, im) 2^-bits, and for every output
+    component total = the sum of |link entry| |projected neighbour| over its 24 products."""
+
+    def __init__(self, U, psi, dims, dagger, ubits=80, bits=200):
+        shape = tuple(dims[::-1])
+        U, psi = U.reshape(shape + (4, 3, 3)), psi.reshape(shape + (4, 3))
+        ur, ui = _ints(U, ubits)
+        pr, pi = _ints(psi, bits)
+        self.bits = ubits + bits
+        re = np.zeros(psi.shape, dtype=object)
+        im = np.zeros(psi.shape, dtype=object)
+        self.total = np.zeros(psi.shape)
+        self.largest = np.zeros(psi.shape[:-2])  # largest real component of a projected neighbour
+        for mu in range(4):
+            ax, gam = 3 - mu, oracle.gamma(mu)
+            edge = [slice(None)] * 4
+            for back in (0, 1):
+                sign = (1 if back else -1) * (-1 if dagger else 1)
+                a = np.eye(4) + sign * gam
+                # (1 +- gamma) psi, in integers and in FP64
+                qr = sum(np.multiply.outer(pr[..., s, :], a[:, s].real.astype(int).astype(object)) -
+                         np.multiply.outer(pi[..., s, :], a[:, s].imag.astype(int).astype(object)) for s in range(4))
+                qi = sum(np.multiply.outer(pi[..., s, :], a[:, s].real.astype(int).astype(object)) +
+                         np.multiply.outer(pr[..., s, :], a[:, s].imag.astype(int).astype(object)) for s in range(4))
+                qr, qi = np.moveaxis(qr, -1, -2), np.moveaxis(qi, -1, -2)
+                q = np.einsum("st,...tc->...sc", a, psi)
+                vr, vi, v = ur[..., mu, :, :], ui[..., mu, :, :], U[..., mu, :, :]
+                if back:  # U^dag psi at the neighbour, then moved here
+                    vr, vi, v = np.swapaxes(vr, -1, -2), -np.swapaxes(vi, -1, -2), np.swapaxes(v, -1, -2).conj()
+                else:
+                    qr, qi, q = (np.roll(x, -1, ax) for x in (qr, qi, q))
+                hr = (vr[..., None, :, :] * qr[..., :, None, :] - vi[..., None, :, :] * qi[..., :, None, :]).sum(-1)
+                hi = (vr[..., None, :, :] * qi[..., :, None, :] + vi[..., None, :, :] * qr[..., :, None, :]).sum(-1)
+                t = (np.abs(v)[..., None, :, :] * np.abs(q)[..., :, None, :]).sum(-1)
+                m = np.maximum(np.abs(q.real), np.abs(q.imag)).max((-2, -1))
+                if back:
+                    hr, hi, t, m = (np.roll(x, 1, ax) for x in (hr, hi, t, m))
+                edge[ax] = 0 if back else dims[mu] - 1
+                hr[tuple(edge)] *= BC[mu]
+                hi[tuple(edge)] *= BC[mu]
+                edge[ax] = slice(None)
+                re, im, self.total = re + hr, im + hi, self.total + t
+                self.largest = np.maximum(self.largest, m)
+        self.re, self.im = re.reshape(-1, 4, 3), im.reshape(-1, 4, 3)
+        self.total = self.total.reshape(-1, 4, 3)
+        self.largest = self.largest.reshape(-1)
+
+    def error(self, got):
+        """got - exact, real and imaginary parts (the differences are exact before they are rounded)."""
+        gr, gi = _ints(got.reshape(-1, 4, 3), self.bits)
+        f = np.frompyfunc(lambda n: float(n) if abs(n) < 2 ** 1000 else float("inf"), 1, 1)
+        scale = 2.0 ** -self.bits
+        return f(gr - self.re).astype(float) * scale, f(gi - self.im).astype(float) * scale
+
+
+def _apply(g, psi, dagger):
+    """The hopping term on both parities: (V, 4, 3) complex, canonical order."""
+    out = torch.zeros_like(psi)
+    for p in (0, 1):
+        i, o = g.field("f64"), g.field("f64")
+        wilson.wl_field_to_internal(g.handle, i, psi, 1 - p, wilson.WL_F64, 1)
+        wilson.wilson_dslash(g.handle, o, i, p, dagger, wilson.WL_F64, 1)
+        wilson.wl_field_to_canonical(g.handle, out, o, p, wilson.WL_F64, 1)
+    return out[0].cpu().numpy()
+
+
+def _cases(dims, links, psi, seed=13, scale=1.0):
+    """(dagger, kernel's result, exact result) for links of a kind."""
+    U = scale * fields.gauge_field(dims, links, seed)
+    with wilson.Gauge(dims, 0.12, U.cuda(), precs=("f64",), bc=BC) as g:
+        for dagger in (0, 1):
+            yield dagger, _apply(g, psi.cuda(), dagger), Exact(U.numpy(), psi[0].numpy(), dims, dagger)
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("kind", ["point", "integers"])
+def test_exact_on_unit_links(dims, shape, kind, monkeypatch):
+    """Sums that binary64 holds exactly come out exact, zeros included: unit links, and one
+    component at one site or small whole numbers everywhere."""
+    monkeypatch.setenv("WL_HOP_BLOCK", str(shape))
+    psi = torch.zeros_like(fields.gaussian_fermion(dims, 1, 1))
+    if kind == "point":
+        psi[0, 5, 1, 2] = 1.0
+    else:
+        psi = torch.view_as_complex(torch.randint(-8, 9, psi.shape + (2,), generator=fields.generator(3)).double())
+    for dagger, got, want in _cases(dims, "unit", psi):
+        re, im = want.error(got)
+        assert not re.any() and not im.any(), dagger
