@@ -57,8 +57,10 @@ extern "C" {
  * WL_F64 fields are IEEE binary64.  The WL_F64 hopping term sums a site's
  * eight neighbours in 64-bit fixed point (units about 2^-56 of the largest
  * neighbour component, more accurate than binary64 sums of terms of that size)
- * when every link entry has a modulus of at most 1.25, as SU(3) links do, and
- * the neighbours lie between 2^-953 and 2^1007; in binary64 otherwise. */
+ * when the links are of about the size of SU(3) matrices (every entry of modulus
+ * at most 1.25, and every row and column zero or with an entry of at least 1/8;
+ * they are held as multiples of 2^-59 then) and the neighbours lie between 2^-953
+ * and 2^1007; in binary64 otherwise. */
 typedef enum { WL_F64 = 0, WL_F32 = 1, WL_F16 = 2, WL_DF64 = 3 } wl_prec;
 
 #define WL_PREC_MASK(p) (1 << (p))

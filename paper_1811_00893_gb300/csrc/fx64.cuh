@@ -22,7 +22,10 @@
 //                that neighbours of like size rarely need another) and the sums
 //                are shifted, rounding to nearest.
 //
-// Room: link entries have modulus <= 1.25 (checked at set-up), so |cross sum|
+// Links that do not fit (fx_link_fits in gauge.cu, at set-up: an entry above 1.25, or
+// rows too small for multiples of 2^-59) keep plain FP64 for the whole lattice.
+//
+// Room: link entries have modulus <= 1.25, so |cross sum|
 // <= 6 (1.25 + 1) 2^59 < 2^63 and |site sum| <= 8 * 3 * 1.25 * sqrt(2) * 2^56 < 2^62.
 // Every step rounds at about 2^-56 of the largest of the neighbours' projected
 // components, where FP64 rounds each of its ~60 dependent operations at 2^-53
@@ -34,6 +37,7 @@ namespace wl {
 
 static constexpr int kFxMinExp = 70, kFxMaxExp = 2030;  // biased exponents the fixed-point path takes
 static constexpr double kFxMaxLink = 1.25;              // largest modulus of a link entry
+static constexpr double kFxMinLink = 0.125;             // least modulus of a row's or column's largest (SU(3): 0.57)
 
 // n_w as (wh, wl) of one real
 __host__ __device__ __forceinline__ void fx_split(double w, int& h, int& l)

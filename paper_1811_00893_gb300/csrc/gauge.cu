@@ -125,16 +125,30 @@ __device__ void store_link_fx(void* base, long long Vh, int d, long long i, cons
     }
 }
 
-// The entries of a link are finite and within the modulus that fixed-point
-// storage has room for (a phase factor leaves the modulus alone); in FP32,
-// whose rounding the bound's margin covers many times.
+// Whether fixed-point storage (multiples of 2^-59) keeps a link as well as FP64
+// does: its entries are finite and within the modulus that the sums have room
+// for, and every row, and every column (a row of the backward link), is zero or has
+// an entry of kFxMinLink, so that 2^-60 is below 2^-57 of it.  (A phase factor
+// leaves the moduli alone.)  Moduli in FP32, whose rounding the bounds' margin covers
+// many times.
 __device__ bool fx_link_fits(const double* u)
 {
-    bool ok = true;
+    bool ok = true, live[6] = {};
+    float top[6] = {};
+#pragma unroll
     for (int k = 0; k < 9; ++k) {
         const float re = (float)u[2 * k], im = (float)u[2 * k + 1];
-        ok &= fmaf(re, re, im * im) <= (float)(kFxMaxLink * kFxMaxLink);
+        const float n = fmaf(re, re, im * im);
+        ok &= n <= (float)(kFxMaxLink * kFxMaxLink);
+        const bool entry = u[2 * k] != 0.0 || u[2 * k + 1] != 0.0;
+        const int row = k / 3, col = 3 + k % 3;
+        top[row] = fmaxf(top[row], n);
+        top[col] = fmaxf(top[col], n);
+        live[row] |= entry;
+        live[col] |= entry;
     }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) ok &= !live[k] || top[k] >= (float)(kFxMinLink * kFxMinLink);
     return ok;
 }
 

@@ -33,7 +33,7 @@ class Exact:
     """The hopping term of one field in integers: out = (re, im) 2^-bits, and for every output
     component total = the sum of |link entry| |projected neighbour| over its 24 products."""
 
-    def __init__(self, U, psi, dims, dagger, ubits=80, bits=200):
+    def __init__(self, U, psi, dims, dagger, ubits=240, bits=200):
         shape = tuple(dims[::-1])
         U, psi = U.reshape(shape + (4, 3, 3)), psi.reshape(shape + (4, 3))
         ur, ui = _ints(U, ubits)
@@ -96,9 +96,9 @@ def _apply(g, psi, dagger):
     return out[0].cpu().numpy()
 
 
-def _cases(dims, links, psi, seed=13, scale=1.0):
-    """(dagger, kernel's result, exact result) for links of a kind."""
-    U = scale * fields.gauge_field(dims, links, seed)
+def _cases(dims, links, psi):
+    """(dagger, kernel's result, exact result) for links of a kind, or given ones."""
+    U = fields.gauge_field(dims, links, 13) if isinstance(links, str) else links
     with wilson.Gauge(dims, 0.12, U.cuda(), precs=("f64",), bc=BC) as g:
         for dagger in (0, 1):
             yield dagger, _apply(g, psi.cuda(), dagger), Exact(U.numpy(), psi[0].numpy(), dims, dagger)
@@ -119,3 +119,28 @@ def test_exact_on_unit_links(dims, shape, kind, monkeypatch):
     for dagger, got, want in _cases(dims, "unit", psi):
         re, im = want.error(got)
         assert not re.any() and not im.any(), dagger
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("kind", ["all 2^-27", "all 2^-40", "all 2^-66", "one link", "a row", "a column", "zeros"])
+def test_small_links(dims, kind):
+    """Links, or rows or columns of them, far below 1 keep all their digits.  Plain FP64 passes each
+    product through at most 16 roundings (projection 1, product sum 6, hop sum 8): 16 * 2^-53 of
+    the sum of the products' moduli (17: second order).  Links that are zero are as good as any."""
+    U = fields.gauge_field(dims, "haar", 13)
+    psi = fields.gaussian_fermion(dims, 1, 11)
+    if kind == "one link":  # and one source, whose only way to site 3 is that link (Ly > 2)
+        U[3, 1] *= 2.0 ** -40
+        psi[:, [s for s in range(psi.shape[1]) if s != 3 + dims[0]]] = 0.0
+    elif kind in ("a row", "a column"):  # of all z links; the sources in one slice, forward of some sites and behind others (Lz > 2)
+        U[:, [0, 1, 3]] = 0.0
+        U[(slice(None), 2) + ((1, slice(None)) if kind == "a row" else (slice(None), 1))] *= 2.0 ** -40
+        psi.reshape(dims[::-1] + (4, 3))[:, [z for z in range(dims[2]) if z != 1]] = 0.0
+    elif kind == "zeros":
+        U[3, 1], U[4, 2, 1], U[5, 0, :, 2] = 0.0, 0.0, 0.0
+    else:
+        U *= 2.0 ** int(kind.split("^")[1])
+    for dagger, got, want in _cases(dims, U, psi):
+        re, im = want.error(got)
+        bound = 17 * 2.0 ** -53 * want.total
+        assert np.all(np.abs(re) <= bound) and np.all(np.abs(im) <= bound), dagger
