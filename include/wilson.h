@@ -54,13 +54,22 @@ extern "C" {
  * mixed-precision solves use it for their intermediate outer residuals,
  * because GB300 executes FP32 many times faster than FP64.  The final
  * convergence check of every solve is WL_F64.
- * WL_F64 fields are IEEE binary64.  The WL_F64 hopping term sums a site's
- * eight neighbours in 64-bit fixed point (units about 2^-56 of the largest
- * neighbour component, more accurate than binary64 sums of terms of that size)
- * when the links are of about the size of SU(3) matrices (every entry of modulus
- * at most 1.25, and every row and column zero or with an entry of at least 1/8;
- * they are held as multiples of 2^-59 then) and the neighbours lie between 2^-953
- * and 2^1007; in binary64 otherwise. */
+ * WL_F64 fields are IEEE binary64.  The WL_F64 hopping term sums a site's eight
+ * neighbours in 64-bit fixed point when the links are of about the size of SU(3)
+ * matrices (every entry of modulus at most 1.25, and every row and column zero or
+ * with an entry of at least 1/8), in binary64 otherwise.  In fixed point:
+ *   - links are held as multiples of 2^-59: an entry below 2^-6 keeps fewer than
+ *     the 53 digits it had, with an error of at most 2^-60;
+ *   - the sum's unit is 2^-55 of a power of two q between a half of and twice the
+ *     largest real component of the site's projected neighbours, and its error
+ *     typically 2.5 of these units (at most 15.5 * 2^-53 q): against exact arithmetic a field's
+ *     rms error is below that of the binary64 kernel;
+ *   - an output component (spin, colour) to which no neighbour contributes q/16
+ *     is computed in binary64 instead, as are sites whose neighbours hold an
+ *     infinity or NaN, exceed 2^1007 or all lie below 2^-953.  So every component
+ *     stays within 2^-45 of the sum of the moduli of its products (with the links as
+ *     held; binary64: 2^-49), and zeros and whole numbers come out exact where
+ *     binary64 holds them. */
 typedef enum { WL_F64 = 0, WL_F32 = 1, WL_F16 = 2, WL_DF64 = 3 } wl_prec;
 
 #define WL_PREC_MASK(p) (1 << (p))

@@ -22,14 +22,18 @@
 //                that neighbours of like size rarely need another) and the sums
 //                are shifted, rounding to nearest.
 //
+// Errors, in units of the site sum: a hop adds at most 6 for its wl xl terms, 1/2
+// for the cross sum, 3/8 for its links' and 1/3 for its neighbour's rounding, a raise
+// of e 1/2: 62 in all, 15.5 2^-53 of 2^(e-1023); typically 2.5.  FP64 rounds each of its
+// ~16 dependent operations at 2^-53 of the partial sum.  What is small next to
+// 2^(e-1023) is computed in FP64 (kFxLeast).
+//
 // Links that do not fit (fx_link_fits in gauge.cu, at set-up: an entry above 1.25, or
 // rows too small for multiples of 2^-59) keep plain FP64 for the whole lattice.
 //
 // Room: link entries have modulus <= 1.25, so |cross sum|
 // <= 6 (1.25 + 1) 2^59 < 2^63 and |site sum| <= 8 * 3 * 1.25 * sqrt(2) * 2^56 < 2^62.
-// Every step rounds at about 2^-56 of the largest of the neighbours' projected
-// components, where FP64 rounds each of its ~60 dependent operations at 2^-53
-// of the partial sum.  A site whose neighbours hold an infinity or NaN, exceed
+// A site whose neighbours hold an infinity or NaN, exceed
 // 2^1007 or all lie below 2^-953 goes through fx_site_general, plain FP64.
 #pragma once
 
@@ -64,14 +68,44 @@ static constexpr long long kFxHalfUnit = 1LL << 30;
 // The site sum: s[(spin * 3 + colour row) * 2 + (0: re, 1: im)]
 struct FxSum {
     long long s[24];
+    // size of the hops' shares, in units of 2^48: the largest |re| or |im| so far of
+    // u0 (low half) and u1 (high half), [x and y hops | z and t hops][colour row]
+    unsigned m[2][3];
     int e;     // biased exponent of the units
     bool bad;  // this site needs fx_site_general
 };
+
+// A component of the site sum keeps its fixed-point value if some hop's share
+// of it reaches 2^-4 of 2^(e-1023) (2^51 units); a component with none is computed
+// in FP64 (fx_site_general), whose rounding follows the size of its own terms.  So a
+// component's error is below 2^-45 of the sum of its products' moduli, wherever
+// those lie below the site's largest.  With neighbours of like size and links that
+// mix the colours one component in 10^13 is that small.  Hopping term of
+// 24^3 x 48: Gaussian field 138 us (136 without the test), a point source's
+// solution 232 us (Haar links) and 294 us (smooth), one spin row 299 us, one colour on
+// unit links 770 us, the plain FP64 kernel 524 us.  Half and a quarter of the
+// limit: the solutions 210 and 178 us, 172 and 140 us.
+static constexpr int kFxLeast = 8;
+
+// The largest of m's halves and |those of a, b|, 16 bits from the top of re and im
+__device__ __forceinline__ unsigned fx_size(unsigned m, long long u0, long long u1)
+{
+    const unsigned p = __byte_perm((unsigned)(u0 >> 32), (unsigned)(u1 >> 32), 0x7632);
+    return __vimax3_s16x2(m, p, ~p);
+}
+// The sizes after the units grew by 2^by
+__device__ __forceinline__ unsigned fx_size_shift(unsigned m, int by)
+{
+    const int k = min(by, 15);
+    return (m >> k) & ((0x7fffu >> k) * 0x10001u);
+}
 
 __device__ __forceinline__ void fx_clear(FxSum& S)
 {
 #pragma unroll
     for (int k = 0; k < 24; ++k) S.s[k] = 0;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) S.m[0][r] = S.m[1][r] = 0;
     S.e = kFxMinExp;
     S.bad = false;
 }
@@ -136,6 +170,11 @@ __device__ __forceinline__ void fx_convert(FxSum& Q, FxHalf& X, const cx<double>
             const long long half = 1LL << (by - 1);
 #pragma unroll
             for (int k = 0; k < 24; ++k) Q.s[k] = (Q.s[k] + half) >> by;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                Q.m[0][r] = fx_size_shift(Q.m[0][r], by);
+                Q.m[1][r] = fx_size_shift(Q.m[1][r], by);
+            }
         }
 #pragma unroll
         for (int q = 0; q < 12; ++q) up[q] += (E - Q.e) << 20;
@@ -190,6 +229,8 @@ __device__ __forceinline__ void fx_row(FxSum& Q, const FxHalf& X, const int4 (&w
     long long *s0 = Q.s + 2 * r, *s1 = s0 + 6, *s2 = s1 + 6, *s3 = s2 + 6;
     fx_add_ik<0>(s0, R[0], R[1]);
     fx_add_ik<0>(s1, R[2], R[3]);
+    if (mu & 2) Q.m[1][r] = fx_size(fx_size(Q.m[1][r], R[0], R[2]), R[1], R[3]);
+    else Q.m[0][r] = fx_size(fx_size(Q.m[0][r], R[0], R[2]), R[1], R[3]);
     if (mu & 1) {
         if (mu & 2) {  // rows 2, 3 += (u0, u1)
             fx_add_ik<0>(s2, R[0], R[1]);
@@ -326,11 +367,13 @@ __device__ __forceinline__ void project_code(cx<T> (&h0)[3], cx<T> (&h1)[3], con
 }
 
 // The site sum in plain FP64 arithmetic (the operations of the LF = 0
-// kernel), for the sites whose neighbours do not share a scale.  half(d, h0, h1)
+// kernel), for components that are small next to the site's scale and for sites
+// whose neighbours do not share a scale.  half(d, h0, h1)
 // gives the projected half spinor of hop d.  A loop, and called rather than
-// inlined: it is rare, and must not cost the fixed-point path registers.
+// inlined: it is rare, and must not cost the fixed-point path registers.  Sets
+// the components of out whose bit (spin * 3 + colour) is in `which`.
 template <bool DAG, typename F>
-__device__ __noinline__ void fx_site_general(double (&out)[24], const void* links, long long lVh, long long li, F half)
+__device__ __noinline__ void fx_site_general(double (&out)[24], unsigned which, const void* links, long long lVh, long long li, F half)
 {
     cx<double> acc[12];
 #pragma unroll
@@ -339,10 +382,17 @@ __device__ __noinline__ void fx_site_general(double (&out)[24], const void* link
     for (int d = 0; d < 8; ++d) {
         cx<double> h0[3], h1[3];
         half(d, h0, h1);
-        bool zero = true;
+        // the colour rows of u0 and u1 that enter components of `which`
+        const unsigned two = which >> (d < 4 ? 9 : 6), three = which >> (d < 4 ? 6 : 9);
+        unsigned n0 = (which | two) & 7u, n1 = (which >> 3 | three) & 7u;
+        bool zero0 = true, zero1 = true;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) zero &= h0[c].re == 0.0 & h0[c].im == 0.0 & h1[c].re == 0.0 & h1[c].im == 0.0;
-        if (zero) continue;
+        for (int c = 0; c < 3; ++c) {
+            zero0 &= h0[c].re == 0.0 & h0[c].im == 0.0;
+            zero1 &= h1[c].re == 0.0 & h1[c].im == 0.0;
+        }
+        if (zero0) n0 = 0;
+        if (zero1) n1 = 0;
         const unsigned code = hop_code(d >> 1);
         const int sflip = ((d & 1) ? DAG == false : DAG == true) ? 0 : 2;
         const int b2 = (code >> 6) & 1, k2 = ((code >> 7) + sflip) & 3;
@@ -350,13 +400,16 @@ __device__ __noinline__ void fx_site_general(double (&out)[24], const void* link
         const int4* p = (const int4*)links + (long long)d * 9 * lVh + li;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
+            if (!((n0 | n1) >> a & 1)) continue;
             cx<double> w[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const int4 t = p[(3 * a + k) * lVh];
                 w[k] = {fx_join(t.x, t.y), fx_join(t.z, t.w)};
             }
-            const cx<double> u0 = dot3(w[0], w[1], w[2], h0), u1 = dot3(w[0], w[1], w[2], h1);
+            cx<double> u0 = {0.0, 0.0}, u1 = {0.0, 0.0};
+            if (n0 >> a & 1) u0 = dot3(w[0], w[1], w[2], h0);
+            if (n1 >> a & 1) u1 = dot3(w[0], w[1], w[2], h1);
             acc[a] = acc[a] + u0;
             acc[3 + a] = acc[3 + a] + u1;
             acc[6 + a] = acc[6 + a] + mul_ik(b2 ? u1 : u0, k2);
@@ -364,26 +417,41 @@ __device__ __noinline__ void fx_site_general(double (&out)[24], const void* link
         }
     }
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-        out[2 * c] = acc[c].re;
-        out[2 * c + 1] = acc[c].im;
-    }
+    for (int c = 0; c < 12; ++c)
+        if (which >> c & 1) {
+            out[2 * c] = acc[c].re;
+            out[2 * c + 1] = acc[c].im;
+        }
 }
 
-// acc = the site sum as FP64
+// acc = the site sum as FP64 (spin rows 2 and 3 take u1, u0 of the x and y hops
+// and u0, u1 of the z and t hops)
 template <bool DAG, typename F>
 __device__ __forceinline__ void fx_finish(cx<double> (&acc)[12], const FxSum& S, const void* links, long long lVh,
                                           long long li, F half)
 {
-    if (S.bad || S.e == kFxMinExp) {  // (nothing above 2^-953: zeros, or too small for fixed point)
-        double g[24];
-        fx_site_general<DAG>(g, links, lVh, li, half);
+    unsigned low = 0;  // components that need FP64
 #pragma unroll
-        for (int c = 0; c < 12; ++c) acc[c] = {g[2 * c], g[2 * c + 1]};
-        return;
+    for (int r = 0; r < 3; ++r) {
+        const unsigned up = __vmaxs2(S.m[0][r], S.m[1][r]);
+        const unsigned down = __vmaxs2(__byte_perm(S.m[0][r], 0, 0x1032), S.m[1][r]);
+        low |= ((up & 0xffffu) < kFxLeast ? 1u : 0u) << r | (up < (unsigned)kFxLeast << 16 ? 8u : 0u) << r |
+               ((down & 0xffffu) < kFxLeast ? 64u : 0u) << r | (down < (unsigned)kFxLeast << 16 ? 512u : 0u) << r;
     }
+    if (S.bad || S.e == kFxMinExp) low = 0xfffu;  // (nothing above 2^-953: zeros, or too small for fixed point)
 #pragma unroll
     for (int c = 0; c < 12; ++c) acc[c] = {fx_value(S.s[2 * c], S.e), fx_value(S.s[2 * c + 1], S.e)};
+    if (low) {
+        double g[24];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            g[2 * c] = acc[c].re;
+            g[2 * c + 1] = acc[c].im;
+        }
+        fx_site_general<DAG>(g, low, links, lVh, li, half);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) acc[c] = {g[2 * c], g[2 * c + 1]};
+    }
 }
 
 // The plain-FP64 path's half spinor of hop d from the local neighbour at n
@@ -541,6 +609,7 @@ __device__ __forceinline__ void fx_site_staged(cx<double> (&acc)[12], const int 
 // Spin row j in s, this thread's parts of spin rows 3 - j and 2 + j in a and b (re, im)
 struct FxPart {
     long long s[2], a[2], b[2];
+    int m[2];  // as FxSum's, of this thread's product: x and y hops, z and t hops
     int e;
     bool bad;
 };
@@ -580,6 +649,8 @@ __device__ __forceinline__ void fx_convert_row(FxPart& Q, int (&xh)[6], int (&xl
             E = Q.e;  // another site's
         }
         const int by = min(E - Q.e, 62);
+        Q.m[0] >>= min(by, 15);
+        Q.m[1] >>= min(by, 15);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             Q.b[k] += fx_partner(Q.a[k]);
@@ -652,6 +723,9 @@ __device__ __forceinline__ void fx_hop_row(FxPart& Q, const cx<double> (&p)[3], 
         D = fx_mad(w[k].w, H[2 * k], D);
     }
     const long long re = A + (B >> 31), im = C + (D >> 31);
+    const int tr = (int)(re >> 48), ti = (int)(im >> 48);
+    int& size = Q.m[MU >> 1];
+    size = max(max(size, max(tr, ~tr)), max(ti, ~ti));
     Q.s[0] += re;
     Q.s[1] += im;
     const long long mm = m;
@@ -680,6 +754,7 @@ __device__ __forceinline__ void fx_site_row(cx<double>& up, cx<double>& down, co
     const int j = lane >> 4;
     FxPart Q;
     Q.s[0] = Q.s[1] = Q.a[0] = Q.a[1] = Q.b[0] = Q.b[1] = 0;
+    Q.m[0] = Q.m[1] = 0;
     Q.e = kFxMinExp;
     Q.bad = false;
     const double2* f = (const double2*)in + 3 * j * Vh;
@@ -725,18 +800,21 @@ __device__ __forceinline__ void fx_site_row(cx<double>& up, cx<double>& down, co
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) Q.b[k] += fx_partner(Q.a[k]);
-    if (Q.bad || Q.e == kFxMinExp) {
-        double g[24];
-        fx_site_general<DAG>(g, links, Vh, li, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
-            fx_general_local<DAG>(d, h0, h1, in, Vh, fx_pick(nb, d));
-        });
-        const int c = 2 * (3 * j + a);
-        up = {g[c], g[c + 1]};
-        down = {g[c + 12], g[c + 13]};
-        return;
-    }
+    const int other = __shfl_xor_sync(0xffffffffu, Q.m[0], 16);  // the x and y hops' share of spin row 2 + j
+    const unsigned above = max(Q.m[0], Q.m[1]) < kFxLeast ? 1u : 0u, below = max(other, Q.m[1]) < kFxLeast ? 64u : 0u;
+    const int c = 3 * j + a;
+    unsigned low = (above | below) << c;
+    if (Q.bad || Q.e == kFxMinExp) low = 65u << c;
     up = {fx_value(Q.s[0], Q.e), fx_value(Q.s[1], Q.e)};
     down = {fx_value(Q.b[0], Q.e), fx_value(Q.b[1], Q.e)};
+    if (low) {
+        double g[24];
+        fx_site_general<DAG>(g, low, links, Vh, li, [=](int d, cx<double>(&h0)[3], cx<double>(&h1)[3]) {
+            fx_general_local<DAG>(d, h0, h1, in, Vh, fx_pick(nb, d));
+        });
+        if (low >> c & 1) up = {g[2 * c], g[2 * c + 1]};
+        if (low >> c & 64) down = {g[2 * c + 12], g[2 * c + 13]};
+    }
 }
 
 }  // namespace wl

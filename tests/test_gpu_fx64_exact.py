@@ -144,3 +144,78 @@ def test_small_links(dims, kind):
         re, im = want.error(got)
         bound = 17 * 2.0 ** -53 * want.total
         assert np.all(np.abs(re) <= bound) and np.all(np.abs(im) <= bound), dagger
+
+
+SMALL = ["colours 1e-6", "colours 1e-10", "colours 1e-20", "spins 1e-9", "imaginary 1e-8", "sites", "components"]
+
+
+def _uneven(dims, kind):
+    """A Gaussian field with parts of it scaled down, or scales all over."""
+    psi, gen = fields.gaussian_fermion(dims, 1, 11), fields.generator(12)
+    if kind.startswith("colours"):
+        psi[..., 1:] *= float(kind.split()[1])
+    elif kind.startswith("spins"):
+        psi[:, :, 1:] *= float(kind.split()[1])
+    elif kind.startswith("imaginary"):
+        psi = torch.complex(psi.real, psi.imag * float(kind.split()[1]))
+    else:
+        n = psi.shape[:2] + ((1, 1) if kind == "sites" else (4, 3))
+        psi *= 10.0 ** (24 * torch.rand(n, generator=gen, dtype=torch.float64) - 12)
+    return psi
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("links", ["unit", "smooth", "haar"])
+@pytest.mark.parametrize("kind", SMALL)
+def test_small_components(dims, shape, links, kind, monkeypatch):
+    """Every component is as accurate as its own terms, also next to larger ones.
+
+    In units of 2^-53 q, q the site's scale, the fixed-point sum is within 15.5 of exact, and a
+    component that keeps it has a contribution of at least q / 16, so within 16 * 15.5 = 248 of its
+    total; projecting (1) and the final rounding (1) add 2, which leaves 250 < 256 = 2^-45 2^53.
+    Components in binary64 pass 16 roundings."""
+    monkeypatch.setenv("WL_HOP_BLOCK", str(shape))
+    for dagger, got, want in _cases(dims, links, _uneven(dims, kind)):
+        re, im = want.error(got)
+        bound = 2.0 ** -45 * want.total
+        assert np.all(np.abs(re) <= bound) and np.all(np.abs(im) <= bound), dagger
+
+
+@pytest.mark.parametrize("kind", ["colours 1e-10", "components"])
+def test_small_components_of_blocks(kind):
+    """The decomposed lattice takes the undivided one's steps, at the cut faces too."""
+    dims = (4, 4, 4, 8)
+    psi = _uneven(dims, kind).cuda()
+    U = fields.gauge_field(dims, "unit", 0).cuda()
+    with wilson.Gauge(dims, 0.12, U, precs=("f64",), bc=BC) as g, \
+            wilson.Decomposition(dims, 0.12, U, (1, 1, 2, 2), precs=("f64",), bc=BC) as dd:
+        want = _apply(g, psi, 0)
+        loc, out = dd.canonical(1), dd.canonical(1)
+        wilson.wl_dd_scatter(dd.handle, loc, psi, 1)
+        for p in (0, 1):
+            di, do = dd.field("f64"), dd.field("f64")
+            for k, (gk, _) in enumerate(dd.blocks):
+                wilson.wl_field_to_internal(gk, di[k], loc[k], 1 - p, wilson.WL_F64, 1)
+            wilson.wilson_dslash_dd(dd.handle, do, di, p, 0, wilson.WL_F64, 1)
+            for k, (gk, _) in enumerate(dd.blocks):
+                wilson.wl_field_to_canonical(gk, out[k], do[k], p, wilson.WL_F64, 1)
+        got = torch.zeros_like(psi)
+        wilson.wl_dd_gather(dd.handle, got, out, 1)
+    assert np.array_equal(got[0].cpu().numpy(), want)
+
+
+def test_one_colour_in_a_batch():
+    """Batched FP64 solves on unit links (links in shared memory): a source of one colour leaves the
+    other colours exactly zero, and the true residual is the oracle's."""
+    dims, kappa = (4, 4, 4, 6), 0.12
+    U = fields.gauge_field(dims, "unit", 0)
+    b = fields.gaussian_fermion(dims, 2, 5)
+    b[..., 1:] = 0.0
+    x = torch.zeros_like(b).cuda()
+    with wilson.Gauge(dims, kappa, U.cuda(), precs=("f64",), bc=BC) as g:
+        wilson.wilson_solve_batch([g.handle], [x], [b.cuda()], [2], wilson.solve_params(tol=1e-10, inner=wilson.WL_F64))
+    x = x.cpu()
+    assert not torch.any(x[..., 1:]) and torch.any(x[..., 0])
+    for r in range(2):
+        assert oracle.true_residual(U.numpy(), b[r].numpy(), x[r].numpy(), dims, BC, kappa) <= 1e-10
