@@ -56,8 +56,9 @@ extern "C" {
  * convergence check of every solve is WL_F64.
  * WL_F64 fields are IEEE binary64.  The WL_F64 hopping term sums a site's eight
  * neighbours in 64-bit fixed point when the links are of about the size of SU(3)
- * matrices (every entry of modulus at most 1.25, and every row and column zero or
- * with an entry of at least 1/8), in binary64 otherwise.  In fixed point:
+ * matrices (every entry of modulus at most 1.25, every row and column zero or
+ * with an entry of at least 1/8, and nonzero entries of modulus below 2^-14 in at
+ * most one link per 1,024), in binary64 otherwise.  In fixed point:
  *   - links are held as multiples of 2^-59: an entry below 2^-6 keeps fewer than
  *     the 53 digits it had, with an error of at most 2^-60;
  *   - the sum's unit is 2^-55 of a power of two q between a half of and twice the
@@ -68,8 +69,8 @@ extern "C" {
  *     is computed in binary64 instead, as are sites whose neighbours hold an
  *     infinity or NaN, exceed 2^1007 or all lie below 2^-953.  So every component
  *     stays within 2^-45 of the sum of the moduli of its products (with the links as
- *     held; binary64: 2^-49), and zeros and whole numbers come out exact where
- *     binary64 holds them. */
+ *     held; binary64: 2^-49), and on links of zeros and ones exact zeros and whole
+ *     numbers come out exact. */
 typedef enum { WL_F64 = 0, WL_F32 = 1, WL_F16 = 2, WL_DF64 = 3 } wl_prec;
 
 #define WL_PREC_MASK(p) (1 << (p))

@@ -29,7 +29,7 @@
 // 2^(e-1023) is computed in FP64 (kFxLeast).
 //
 // Links that do not fit (fx_link_fits in gauge.cu, at set-up: an entry above 1.25, or
-// rows too small for multiples of 2^-59) keep plain FP64 for the whole lattice.
+// rows or entries too small for multiples of 2^-59) keep plain FP64 for the whole lattice.
 //
 // Room: link entries have modulus <= 1.25, so |cross sum|
 // <= 6 (1.25 + 1) 2^59 < 2^63 and |site sum| <= 8 * 3 * 1.25 * sqrt(2) * 2^56 < 2^62.
@@ -42,6 +42,12 @@ namespace wl {
 static constexpr int kFxMinExp = 70, kFxMaxExp = 2030;  // biased exponents the fixed-point path takes
 static constexpr double kFxMaxLink = 1.25;              // largest modulus of a link entry
 static constexpr double kFxMinLink = 0.125;             // least modulus of a row's or column's largest (SU(3): 0.57)
+// Nonzero entries of modulus below 2^-14 have an error above 2^-45 of themselves.
+// One matters where no other link of a site carries the same component, as on
+// links near 1: links with such entries are at most one in 1,024 (Haar links: one
+// in 10^7; smooth ones of width 0.3: one in 10^6).
+static constexpr double kFxTinyLink = 0x1p-14;
+static constexpr int kFxTinyShare = 1024;
 
 // n_w as (wh, wl) of one real
 __host__ __device__ __forceinline__ void fx_split(double w, int& h, int& l)

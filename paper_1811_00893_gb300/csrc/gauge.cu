@@ -130,10 +130,11 @@ __device__ void store_link_fx(void* base, long long Vh, int d, long long i, cons
 // for, and every row, and every column (a row of the backward link), is zero or has
 // an entry of kFxMinLink, so that 2^-60 is below 2^-57 of it.  (A phase factor
 // leaves the moduli alone.)  Moduli in FP32, whose rounding the bounds' margin covers
-// many times.
-__device__ bool fx_link_fits(const double* u)
+// many times.  flag[0] is set for a link that does not fit, flag[1] counts those with
+// a nonzero entry below kFxTinyLink.
+__device__ void fx_check_link(const double* u, int* flag)
 {
-    bool ok = true, live[6] = {};
+    bool ok = true, tiny = false, live[6] = {};
     float top[6] = {};
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
@@ -141,6 +142,7 @@ __device__ bool fx_link_fits(const double* u)
         const float n = fmaf(re, re, im * im);
         ok &= n <= (float)(kFxMaxLink * kFxMaxLink);
         const bool entry = u[2 * k] != 0.0 || u[2 * k + 1] != 0.0;
+        tiny |= entry && n < (float)(kFxTinyLink * kFxTinyLink);
         const int row = k / 3, col = 3 + k % 3;
         top[row] = fmaxf(top[row], n);
         top[col] = fmaxf(top[col], n);
@@ -149,7 +151,8 @@ __device__ bool fx_link_fits(const double* u)
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) ok &= !live[k] || top[k] >= (float)(kFxMinLink * kFxMinLink);
-    return ok;
+    if (!ok) flag[0] = 1;
+    if (tiny) atomicAdd(&flag[1], 1);
 }
 
 // The same over all links of a lattice: a block of a decomposition takes the
@@ -157,7 +160,7 @@ __device__ bool fx_link_fits(const double* u)
 __global__ void __launch_bounds__(256) check_links_kernel(const double* __restrict__ U, long long nlinks, int* flag)
 {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nlinks; k += (long long)gridDim.x * blockDim.x)
-        if (!fx_link_fits(U + 18 * k)) *flag = 1;
+        fx_check_link(U + 18 * k, flag);
 }
 
 struct BC {
@@ -203,7 +206,7 @@ __global__ void build_links_kernel(void* out, const double* __restrict__ U, Geom
         cx<double> w[9];
         // forward: phi^[x_mu = L-1] U_mu(x)
         const double* u = U + (s * 4 + mu) * 18;
-        if (FX && !fx_link_fits(u)) *flag = 1;
+        if (FX && flag) fx_check_link(u, flag);
         double pr = 1.0, pi = 0.0;
         if (c[mu] == G.L[mu] - 1) { pr = bc.re[mu]; pi = bc.im[mu]; }
         for (int k = 0; k < 9; ++k) {
@@ -633,9 +636,10 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
                 }
                 if (prec == WL_F64) {  // fixed point, until a link turns out not to fit (below)
                     int* flag = (int*)((char*)g->links[prec][p] + link_field_bytes(prec, g->geo.Vh));
-                    cudaMemsetAsync(flag, 0, sizeof(int), s);
-                    build_links_kernel<WL_F64, true><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p, flag);
-                    if (global != local)
+                    const bool whole = global == local;  // (each link is checked once: by its site's parity, or below)
+                    cudaMemsetAsync(flag, 0, 2 * sizeof(int), s);
+                    build_links_kernel<WL_F64, true><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p, whole ? flag : nullptr);
+                    if (!whole && p == 0)
                         check_links_kernel<<<8u * (unsigned)g->num_sms, 256, 0, s>>>(U, 8 * pl.gl.Vh, flag);
                 }
                 else if (prec == WL_F32) build_links_kernel<WL_F32><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p);
@@ -712,12 +716,13 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
                 rc = set_error(WL_ERR_ARG, "WL_LINKS_R8 needs SU(3) links (unitary, det 1, to 1e-6)");
             if (rc != WL_OK) break;
         }
-        int flags[2] = {0, 0};
+        int flags[2][2] = {};
         for (int p = 0; p < 2; ++p)
-            cudaMemcpyAsync(&flags[p], (char*)g->links[WL_F64][p] + link_field_bytes(WL_F64, g->geo.Vh), sizeof(int),
+            cudaMemcpyAsync(flags[p], (char*)g->links[WL_F64][p] + link_field_bytes(WL_F64, g->geo.Vh), 2 * sizeof(int),
                             cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(WL_ERR_CUDA, "link build failed"); break; }
-        g->fx64 = !flags[0] && !flags[1];
+        g->fx64 = !flags[0][0] && !flags[1][0] &&
+                  ((long long)flags[0][1] + flags[1][1]) * kFxTinyShare <= 8 * pl.gl.Vh;
         if (!g->fx64)  // plain FP64 links instead
             for (int p = 0; p < 2; ++p) {
                 build_links_kernel<WL_F64><<<grid, block, 0, s>>>(g->links[WL_F64][p], U, g->geo, pl, bc, p);

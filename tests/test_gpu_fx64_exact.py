@@ -96,6 +96,22 @@ def _apply(g, psi, dagger):
     return out[0].cpu().numpy()
 
 
+def _apply_blocks(dd, psi):
+    """The same on a decomposed lattice."""
+    loc, out = dd.canonical(1), dd.canonical(1)
+    wilson.wl_dd_scatter(dd.handle, loc, psi, 1)
+    for p in (0, 1):
+        di, do = dd.field("f64"), dd.field("f64")
+        for k, (gk, _) in enumerate(dd.blocks):
+            wilson.wl_field_to_internal(gk, di[k], loc[k], 1 - p, wilson.WL_F64, 1)
+        wilson.wilson_dslash_dd(dd.handle, do, di, p, 0, wilson.WL_F64, 1)
+        for k, (gk, _) in enumerate(dd.blocks):
+            wilson.wl_field_to_canonical(gk, out[k], do[k], p, wilson.WL_F64, 1)
+    got = torch.zeros_like(psi)
+    wilson.wl_dd_gather(dd.handle, got, out, 1)
+    return got[0].cpu().numpy()
+
+
 def _cases(dims, links, psi):
     """(dagger, kernel's result, exact result) for links of a kind, or given ones."""
     U = fields.gauge_field(dims, links, 13) if isinstance(links, str) else links
@@ -191,18 +207,28 @@ def test_small_components_of_blocks(kind):
     with wilson.Gauge(dims, 0.12, U, precs=("f64",), bc=BC) as g, \
             wilson.Decomposition(dims, 0.12, U, (1, 1, 2, 2), precs=("f64",), bc=BC) as dd:
         want = _apply(g, psi, 0)
-        loc, out = dd.canonical(1), dd.canonical(1)
-        wilson.wl_dd_scatter(dd.handle, loc, psi, 1)
-        for p in (0, 1):
-            di, do = dd.field("f64"), dd.field("f64")
-            for k, (gk, _) in enumerate(dd.blocks):
-                wilson.wl_field_to_internal(gk, di[k], loc[k], 1 - p, wilson.WL_F64, 1)
-            wilson.wilson_dslash_dd(dd.handle, do, di, p, 0, wilson.WL_F64, 1)
-            for k, (gk, _) in enumerate(dd.blocks):
-                wilson.wl_field_to_canonical(gk, out[k], do[k], p, wilson.WL_F64, 1)
-        got = torch.zeros_like(psi)
-        wilson.wl_dd_gather(dd.handle, got, out, 1)
-    assert np.array_equal(got[0].cpu().numpy(), want)
+        got = _apply_blocks(dd, psi)
+    assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("blocks", [1, 2])
+def test_links_near_one(blocks):
+    """Links 1 + O(1e-8): the way from one colour to another is worth 1e-8, and keeps its digits
+    (test_small_components' bound), on the whole lattice and on blocks."""
+    dims = (4, 4, 4, 8)
+    U = fields.gauge_field(dims, "smooth", 13, eps=1e-8)
+    psi = fields.gaussian_fermion(dims, 1, 11)
+    psi[..., 1:] = 0.0
+    if blocks == 1:
+        with wilson.Gauge(dims, 0.12, U.cuda(), precs=("f64",), bc=BC) as g:
+            got = _apply(g, psi.cuda(), 0)
+    else:
+        with wilson.Decomposition(dims, 0.12, U.cuda(), (1, 1, 1, blocks), precs=("f64",), bc=BC) as dd:
+            got = _apply_blocks(dd, psi.cuda())
+    want = Exact(U.numpy(), psi[0].numpy(), dims, 0)
+    re, im = want.error(got)
+    bound = 2.0 ** -45 * want.total
+    assert np.all(np.abs(re) <= bound) and np.all(np.abs(im) <= bound)
 
 
 def test_one_colour_in_a_batch():
