@@ -399,8 +399,20 @@ static int persistent_grid(const BatchCtx& C, int lanes)
     return per_sm * C.sms;
 }
 
+static void launch_update_p(const BatchCtx& C, cudaStream_t s)
+{
+    const BatchArgs a = args_of(C);
+    const dim3 grid((unsigned)C.max_chunks, (unsigned)C.nsys);
+    if (C.P == WL_F64) batch_update_p_kernel<WL_F64><<<grid, kBlock, 0, s>>>(a);
+    else if (C.P == WL_F32) batch_update_p_kernel<WL_F32><<<grid, kBlock, 0, s>>>(a);
+    else batch_update_p_kernel<WL_F16><<<grid, kBlock, 0, s>>>(a);
+}
+
 // Pick the right-hand-side lanes of the persistent kernel by timing the
-// first hopping operation (tmp = H p, which only writes a temporary).
+// first hopping operation (tmp = H p, which only writes a temporary).  This is
+// before the first iteration of a round, which leaves p unwritten until that
+// iteration sets p = r: so p = r is set here too, and the timed launches see
+// the iteration's values (FP64 takes longer on zeros or leftovers, fx64.cuh).
 static int tune_batch(BatchCtx& C, cudaStream_t s)
 {
     int maxr = 1;
@@ -418,6 +430,10 @@ static int tune_batch(BatchCtx& C, cudaStream_t s)
     WL_CUDA(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_l = C.lanes;
+    launch_update_p(C, s);
+    WL_CHECK_LAUNCH(0.0);
+    const bool verbose = getenv("WL_AUTOTUNE_VERBOSE") != nullptr;
+    if (verbose) fprintf(stderr, "[wl autotune] batch hop p%d lattices %d systems %d:", C.P, C.nlat, C.nsys);
     for (int l : cand) {
         C.lanes = l;
         C.grid = persistent_grid(C, l);
@@ -434,11 +450,13 @@ static int tune_batch(BatchCtx& C, cudaStream_t s)
             cudaEventElapsedTime(&ms, e0, e1);
             t = std::min(t, ms);
         }
+        if (verbose) fprintf(stderr, " %d:%.1fus", l, t * 1e3f);
         if (t < best) {
             best = t;
             best_l = l;
         }
     }
+    if (verbose) fprintf(stderr, " -> %d\n", best_l);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     C.lanes = best_l;
@@ -454,18 +472,15 @@ static int enqueue_batch_iteration(const BatchCtx& C, cudaStream_t s)
     auto vec = [&](int which) -> int {
         switch (C.P) {
             case WL_F64:
-                if (which == 0) batch_update_p_kernel<WL_F64><<<vgrid, kBlock, 0, s>>>(a);
-                else if (which == 1) batch_update_s_kernel<WL_F64><<<vgrid, kBlock, 0, s>>>(a);
+                if (which == 1) batch_update_s_kernel<WL_F64><<<vgrid, kBlock, 0, s>>>(a);
                 else batch_update_xr_kernel<WL_F64, WL_F64><<<vgrid, kBlock, 0, s>>>(a);
                 break;
             case WL_F32:
-                if (which == 0) batch_update_p_kernel<WL_F32><<<vgrid, kBlock, 0, s>>>(a);
-                else if (which == 1) batch_update_s_kernel<WL_F32><<<vgrid, kBlock, 0, s>>>(a);
+                if (which == 1) batch_update_s_kernel<WL_F32><<<vgrid, kBlock, 0, s>>>(a);
                 else batch_update_xr_kernel<WL_F32, WL_F32><<<vgrid, kBlock, 0, s>>>(a);
                 break;
             default:
-                if (which == 0) batch_update_p_kernel<WL_F16><<<vgrid, kBlock, 0, s>>>(a);
-                else if (which == 1) batch_update_s_kernel<WL_F16><<<vgrid, kBlock, 0, s>>>(a);
+                if (which == 1) batch_update_s_kernel<WL_F16><<<vgrid, kBlock, 0, s>>>(a);
                 else batch_update_xr_kernel<WL_F16, WL_F32><<<vgrid, kBlock, 0, s>>>(a);
                 break;
         }
@@ -480,7 +495,8 @@ static int enqueue_batch_iteration(const BatchCtx& C, cudaStream_t s)
         if (op & 1) WL_CHECK_LAUNCH(0.0);
         return WL_OK;
     };
-    WL_TRY(vec(0));
+    launch_update_p(C, s);
+    WL_CHECK_LAUNCH(per_op);
     WL_TRY(hop(0));
     WL_TRY(hop(1));
     WL_TRY(vec(1));
