@@ -162,6 +162,63 @@ def test_small_links(dims, kind):
         assert np.all(np.abs(re) <= bound) and np.all(np.abs(im) <= bound), dagger
 
 
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("links", ["haar", "smooth"])
+def test_error_of_a_field(dims, shape, links, monkeypatch):
+    """Gaussian fields: every component within the steps' bound, and the root mean square of the errors
+    no larger than that of the plain FP64 kernels (the links doubled, result halved: exact).
+
+    Bound per component, in units of 2^-53 m, m the largest real component of the site's projected
+    neighbours (the scale q is at most 2 m): the sum's 15.5 q are 31, projecting rounds eight times six
+    products of a row of norm 1 by 2^-53 m (8 sqrt(6) < 20), and the sum, below 8 sqrt(6) m, is
+    rounded once more (20): 71."""
+    monkeypatch.setenv("WL_HOP_BLOCK", str(shape))
+    psi = fields.gaussian_fermion(dims, 1, 11)
+    U = fields.gauge_field(dims, links, 13)
+    squares = np.zeros(2)
+    for (dagger, got, want), (_, double, _) in zip(_cases(dims, U, psi), _cases(dims, 2 * U, psi)):
+        bound = 71 * 2.0 ** -53 * want.largest[:, None, None]
+        for k, x in enumerate((got, double / 2)):
+            re, im = want.error(x)
+            squares[k] += (re ** 2).sum() + (im ** 2).sum()
+            assert k or (np.all(np.abs(re) <= bound) and np.all(np.abs(im) <= bound)), dagger
+    assert squares[0] <= squares[1], np.sqrt(squares)
+
+
+@pytest.mark.parametrize("dims", DIMS[:2])
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_six_threads_per_site_on_a_partial_tile(dims, nrhs, monkeypatch):
+    """D, M_ee and their daggers on 8 and 24 sites a parity, bit for bit those of one thread per site;
+    FP64 solves (the reducing forms) to the oracle's residual."""
+    kappa = 0.12
+    U = fields.gauge_field(dims, "haar", 13)
+    psi = fields.gaussian_fermion(dims, nrhs, 11).cuda()
+    outs = {}
+    for shape in SHAPES:
+        monkeypatch.setenv("WL_HOP_BLOCK", str(shape))
+        with wilson.Gauge(dims, kappa, U.cuda(), precs=("f64",), bc=BC) as g:
+            fb = wilson.wl_field_bytes(g.handle, wilson.WL_F64, 1)
+            full = torch.empty(2 * nrhs * fb, dtype=torch.uint8, device="cuda")
+            for k in range(2 * nrhs):
+                wilson.wl_field_to_internal(g.handle, full[k * fb:(k + 1) * fb], psi[k // 2:k // 2 + 1], k % 2, wilson.WL_F64, 1)
+            even = g.field("f64", nrhs)
+            wilson.wl_field_to_internal(g.handle, even, psi, 0, wilson.WL_F64, nrhs)
+            for eo, x in ((0, full), (1, even)):
+                for dagger in (0, 1):
+                    out = torch.zeros_like(x)
+                    wilson.wilson_mult(g.handle, out, x, eo, dagger, wilson.WL_F64, nrhs)
+                    outs.setdefault((eo, dagger), []).append(out.cpu())
+            for eo in (False, True):
+                x = torch.zeros_like(psi)
+                wilson.wilson_solve(g.handle, x, psi, nrhs, wilson.solve_params(tol=1e-10, eo=eo, inner=wilson.WL_F64))
+                for r in range(nrhs):
+                    tr = oracle.true_residual(U.numpy(), psi[r].cpu().numpy(), x[r].cpu().numpy(), dims, BC, kappa)
+                    assert tr <= 1e-10, (shape, eo, r)
+    for key, (one, six) in outs.items():
+        assert torch.equal(one, six), key
+
+
 SMALL = ["colours 1e-6", "colours 1e-10", "colours 1e-20", "spins 1e-9", "imaginary 1e-8", "sites", "components"]
 
 
