@@ -114,9 +114,10 @@ __device__ __forceinline__ void store_link<WL_F16>(void* base, long long Vh, int
 }
 
 // FP64 links as fixed point (LF = 3 of the hopping kernels)
-__device__ void store_link_fx(void* base, long long Vh, int d, long long i, const cx<double> (&w)[9])
+__device__ __forceinline__ void store_link_fx(void* base, long long Vh, int d, long long i, const cx<double> (&w)[9])
 {
     int4* p = (int4*)base + (long long)d * 9 * Vh;
+#pragma unroll
     for (int k = 0; k < 9; ++k) {
         int4 t;
         fx_split(w[k].re, t.x, t.y);
@@ -129,19 +130,27 @@ __device__ void store_link_fx(void* base, long long Vh, int d, long long i, cons
 // does: its entries are finite and within the modulus that the sums have room
 // for, and every row, and every column (a row of the backward link), is zero or has
 // an entry of kFxMinLink, so that 2^-60 is below 2^-57 of it.  (A phase factor
-// leaves the moduli alone.)  Moduli in FP32, whose rounding the bounds' margin covers
-// many times.  flag[0] is set for a link that does not fit, flag[1] counts those with
-// a nonzero entry below kFxTinyLink.
-__device__ void fx_check_link(const double* u, int* flag)
+// leaves the moduli alone.)  Moduli in FP32, from the encodings cut to 24 bits (below
+// 2^-126: 0; from 2^127: infinity), which the bounds' margin covers many times.
+// flag[0] is set for a link that does not fit, flag[1] counts those with a nonzero
+// entry below kFxTinyLink.
+__device__ __forceinline__ void fx_check_link(const double (&u)[18], int* flag)
 {
     bool ok = true, tiny = false, live[6] = {};
     float top[6] = {};
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const float re = (float)u[2 * k], im = (float)u[2 * k + 1];
+        unsigned bits[2];  // |re|, |im| in FP32
+        bool entry = false;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const unsigned hi = (unsigned)__double2hiint(u[2 * k + c]) & 0x7fffffffu, lo = (unsigned)__double2loint(u[2 * k + c]);
+            bits[c] = hi < (897u << 20) ? 0u : hi >= (1150u << 20) ? 0x7f800000u : (hi - (896u << 20)) << 3 | lo >> 29;
+            entry |= (hi | lo) != 0;
+        }
+        const float re = __uint_as_float(bits[0]), im = __uint_as_float(bits[1]);
         const float n = fmaf(re, re, im * im);
         ok &= n <= (float)(kFxMaxLink * kFxMaxLink);
-        const bool entry = u[2 * k] != 0.0 || u[2 * k + 1] != 0.0;
         tiny |= entry && n < (float)(kFxTinyLink * kFxTinyLink);
         const int row = k / 3, col = 3 + k % 3;
         top[row] = fmaxf(top[row], n);
@@ -159,8 +168,12 @@ __device__ void fx_check_link(const double* u, int* flag)
 // form that the whole lattice's links allow.
 __global__ void __launch_bounds__(256) check_links_kernel(const double* __restrict__ U, long long nlinks, int* flag)
 {
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nlinks; k += (long long)gridDim.x * blockDim.x)
-        fx_check_link(U + 18 * k, flag);
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nlinks; k += (long long)gridDim.x * blockDim.x) {
+        double u[18];
+#pragma unroll
+        for (int q = 0; q < 18; ++q) u[q] = U[18 * k + q];
+        fx_check_link(u, flag);
+    }
 }
 
 struct BC {
@@ -205,7 +218,9 @@ __global__ void build_links_kernel(void* out, const double* __restrict__ U, Geom
     for (int mu = 0; mu < 4; ++mu) {
         cx<double> w[9];
         // forward: phi^[x_mu = L-1] U_mu(x)
-        const double* u = U + (s * 4 + mu) * 18;
+        double u[18];
+#pragma unroll
+        for (int q = 0; q < 18; ++q) u[q] = U[(s * 4 + mu) * 18 + q];
         if (FX && flag) fx_check_link(u, flag);
         double pr = 1.0, pi = 0.0;
         if (c[mu] == G.L[mu] - 1) { pr = bc.re[mu]; pi = bc.im[mu]; }
@@ -635,9 +650,9 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
                     break;
                 }
                 if (prec == WL_F64) {  // fixed point, until a link turns out not to fit (below)
-                    int* flag = (int*)((char*)g->links[prec][p] + link_field_bytes(prec, g->geo.Vh));
+                    int* flag = (int*)((char*)g->links[prec][0] + link_field_bytes(prec, g->geo.Vh));
                     const bool whole = global == local;  // (each link is checked once: by its site's parity, or below)
-                    cudaMemsetAsync(flag, 0, 2 * sizeof(int), s);
+                    if (p == 0) cudaMemsetAsync(flag, 0, 2 * sizeof(int), s);
                     build_links_kernel<WL_F64, true><<<grid, block, 0, s>>>(g->links[prec][p], U, g->geo, pl, bc, p, whole ? flag : nullptr);
                     if (!whole && p == 0)
                         check_links_kernel<<<8u * (unsigned)g->num_sms, 256, 0, s>>>(U, 8 * pl.gl.Vh, flag);
@@ -716,18 +731,16 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
                 rc = set_error(WL_ERR_ARG, "WL_LINKS_R8 needs SU(3) links (unitary, det 1, to 1e-6)");
             if (rc != WL_OK) break;
         }
-        int flags[2][2] = {};
-        for (int p = 0; p < 2; ++p)
-            cudaMemcpyAsync(flags[p], (char*)g->links[WL_F64][p] + link_field_bytes(WL_F64, g->geo.Vh), 2 * sizeof(int),
-                            cudaMemcpyDeviceToHost, s);
+        int flags[2] = {};
+        cudaMemcpyAsync(flags, (char*)g->links[WL_F64][0] + link_field_bytes(WL_F64, g->geo.Vh), sizeof flags,
+                        cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(WL_ERR_CUDA, "link build failed"); break; }
-        g->fx64 = !flags[0][0] && !flags[1][0] &&
-                  ((long long)flags[0][1] + flags[1][1]) * kFxTinyShare <= 8 * pl.gl.Vh;
-        if (!g->fx64)  // plain FP64 links instead
-            for (int p = 0; p < 2; ++p) {
-                build_links_kernel<WL_F64><<<grid, block, 0, s>>>(g->links[WL_F64][p], U, g->geo, pl, bc, p);
-                count_launch(1, (double)g->geo.Vh * (8 * 144.0 + link_field_bytes(WL_F64, 1)));
-            }
+        g->fx64 = !flags[0] && (long long)flags[1] * kFxTinyShare <= 8 * pl.gl.Vh;
+        if (g->fx64) break;
+        for (int p = 0; p < 2; ++p) {  // plain FP64 links instead
+            build_links_kernel<WL_F64><<<grid, block, 0, s>>>(g->links[WL_F64][p], U, g->geo, pl, bc, p);
+            count_launch(1, (double)g->geo.Vh * (8 * 144.0 + link_field_bytes(WL_F64, 1)));
+        }
         // the link build reads U: finish before returning so U may be freed
         if (cudaStreamSynchronize(s) != cudaSuccess) { rc = set_error(WL_ERR_CUDA, "link build failed"); break; }
     } while (0);

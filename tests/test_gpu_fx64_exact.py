@@ -137,6 +137,26 @@ def test_exact_on_unit_links(dims, shape, kind, monkeypatch):
         assert not re.any() and not im.any(), dagger
 
 
+def test_links_round_to_nearest():
+    """Small off-diagonal entries of x links come out as the nearest multiples of 2^-59 (ties to even):
+    a constant source of colour 1 reaches colour 0 through them alone, and components that small
+    next to colour 1 are computed from the links as held."""
+    dims = (4, 4, 4, 4)
+    V = fields.volume(dims)
+    psi = torch.zeros_like(fields.gaussian_fermion(dims, 1, 1))
+    psi[..., 0, 1] = 1.0
+    gen = np.random.default_rng(5)
+    many = gen.uniform(2.0 ** -13, 2.0 ** -6, V) * gen.choice([-1.0, 1.0], V)
+    ties = (gen.integers(2 ** 47, 2 ** 51, V) + 0.5) * 2.0 ** -59 * gen.choice([-1.0, 1.0], V)
+    few = [k * 2.0 ** -60 for k in (1, 1 + 2.0 ** -52, 1.5, 2, 3, 5, -1, -3, 2.0 ** -3)] + [5e-324, 1e-300]
+    for values in [many, ties, np.concatenate([many[:V - 1], [0.0]])] + [np.array([0.0] * 7 + [v] + [0.0] * (V - 8)) for v in few]:
+        U = fields.gauge_field(dims, "unit", 0)
+        U[:, 0, 0, 1] = torch.from_numpy(values).to(U.dtype)
+        with wilson.Gauge(dims, 0.12, U.cuda(), precs=("f64",), bc=BC) as g:
+            got = _apply(g, psi.cuda(), 0)[:, 0, 0]
+        assert np.array_equal(got.real, np.rint(values * 2.0 ** 59) * 2.0 ** -59) and not got.imag.any()
+
+
 @pytest.mark.parametrize("dims", DIMS)
 @pytest.mark.parametrize("kind", ["all 2^-27", "all 2^-40", "all 2^-66", "one link", "a row", "a column", "zeros"])
 def test_small_links(dims, kind):
