@@ -50,10 +50,12 @@ extern "C" {
 
 /* Storage precisions.  WL_DF64 stores each real as an unevaluated sum of two
  * FP32 numbers (hi + lo, a 48-bit significand) in FP64-sized fields and
- * computes with FP32 instructions (~2^-44 relative rounding per operation);
- * mixed-precision solves use it for their intermediate outer residuals,
- * because GB300 executes FP32 many times faster than FP64.  The final
- * convergence check of every solve is WL_F64.
+ * computes with FP32 instructions (~2^-44 relative rounding per operation).
+ * Mixed-precision solves take their intermediate outer residuals in WL_F64 with
+ * fixed-point links (below), and in WL_DF64, whose FP32 instructions GB300
+ * executes many times faster than FP64's, where the links do not fit fixed point,
+ * with a clover term and on decomposed lattices.  The final convergence check
+ * of every solve is WL_F64.
  * WL_F64 fields are IEEE binary64.  The WL_F64 hopping term sums a site's eight
  * neighbours in 64-bit fixed point when the links are of about the size of SU(3)
  * matrices (every entry of modulus at most 1.25, every row and column zero or
@@ -63,8 +65,8 @@ extern "C" {
  *     the 53 digits it had, with an error of at most 2^-60;
  *   - the sum's unit is 2^-55 of a power of two q between a half of and twice the
  *     largest real component of the site's projected neighbours, and its error
- *     typically 2.5 of these units (at most 15.5 * 2^-53 q): against exact arithmetic a field's
- *     rms error is below that of the binary64 kernel;
+ *     typically 2.5 of these units (at most 15.5 * 2^-53 q): a Gaussian field's rms
+ *     error against exact arithmetic is below that of the binary64 kernel;
  *   - an output component (spin, colour) to which no neighbour contributes q/16
  *     is computed in binary64 instead, as are sites whose neighbours hold an
  *     infinity or NaN, exceed 2^1007 or all lie below 2^-953.  So every component
@@ -127,7 +129,8 @@ typedef struct wl_gauge_s* wl_gauge;
  * V*4*9 complex, Sec. 2 "link variable").  prec_mask selects which internal
  * link copies to build (WL_PREC_MASK(WL_F32) | ...); FP64 links are always
  * built because the final residual of every solve is FP64, and df64 links
- * whenever FP32 or FP16 is requested (the outer corrections use them).  Returns
+ * whenever FP32 or FP16 is requested (WL_DF64 calls on such an object use them,
+ * and the outer corrections named at wl_prec).  Returns
  * WL_ERR_ARG for odd or small extents, |phi| != 1 or a NULL pointer.  U is
  * only read during the call (stream-ordered) and may be freed afterwards. */
 int wl_gauge_create(wl_gauge* g, const wl_lattice* lat, const double* U, int prec_mask,
@@ -383,7 +386,8 @@ typedef struct {
  * (at most 16); faces of other blocks and the global sums go through `tr`
  * (required when count is below the number of blocks, optional otherwise;
  * copied, and used until wl_dd_destroy).  U is the whole lattice's canonical
- * gauge field on this device (its held blocks and their faces are read). */
+ * gauge field on this device (its held blocks and their faces become links; all
+ * of it is looked at for the form of the FP64 links, which is one for all blocks). */
 int wl_dd_create_part(wl_dd* dd, const wl_lattice* lat, const int grid[4], int first, int count,
                       const double* U, int prec_mask, const wl_dd_transport* tr, void* stream);
 

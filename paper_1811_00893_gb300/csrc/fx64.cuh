@@ -50,9 +50,10 @@ static constexpr double kFxTinyLink = 0x1p-14;
 static constexpr int kFxTinyShare = 1024;
 
 // n_w as (wh, wl) of one real, |w| < 2: the 53-bit significand shifted to units of
-// 2^-59, rounded to nearest, ties to even.  Integer operations: a multiplication
-// and a conversion per real on the FP64 pipe, with the moduli of the check in FP64
-// too, take the kernel of one parity of 32^3 x 64 from 630 us to 1.3 ms.
+// 2^-59, rounded to nearest, ties to even.  Integer operations: with a multiplication
+// and a conversion per real on the FP64 pipe, the check's moduli there too and the link
+// in local memory, creating a gauge object of 32^3 x 64 in FP64 and FP32 took 6.1 ms, so
+// 4.56 (4.42 with FP64 links).
 __device__ __forceinline__ void fx_split(double w, int& h, int& l)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(w);

@@ -627,7 +627,8 @@ int gauge_create(wl_gauge* out, const wl_lattice* local, const wl_lattice* globa
     pl.gl = make_geom(global->dims);
     for (int k = 0; k < 4; ++k) pl.o[k] = origin ? origin[k] : 0;
     g->prec_mask = (prec_mask & WL_PREC_ALL) | WL_PREC_MASK(WL_F64);
-    // the outer residual corrections of mixed-precision solves run in df64
+    // df64 links come with FP32 and FP16: WL_DF64 calls, clover and decomposed
+    // solves, and links that do not fit fixed point read them, after U is gone
     if (g->prec_mask & (WL_PREC_MASK(WL_F32) | WL_PREC_MASK(WL_F16)))
         g->prec_mask |= WL_PREC_MASK(WL_DF64);
     int rc = WL_OK;

@@ -126,6 +126,9 @@ __global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_kerne
 // ahead (all of them at once: 533 us), in FP16, whose arithmetic per byte is
 // higher, all at once (one ahead: 424 us).  D-hat of 24^3 x 48 with 12
 // right-hand sides: FP32 534 us without this prefetch, 510 us with it; FP16 411 us.
+// The two the other way round, from 16^3 x 32 with 2 right-hand sides to 24^3 x 48
+// with 32 and 32^3 x 64 with 3 and 8 (nine sizes and counts): FP32 0.99 to 1.09
+// of this, FP16 0.985 to 1.04; only 16^3 x 32 with 12 in FP16 gains more than 1 %.
 // Prefetching the links of a tile 304 or 1,216 tiles on: FP32 519 and 533 us.
 template <int P, bool DAG, bool DOT, int CL, int LF>
 __global__ void __launch_bounds__(256, (MinBlocks<P, DOT, LF>::value)) hop_mrhs_kernel(const HopArgs A, int nrhs)
@@ -275,14 +278,15 @@ __global__ void __launch_bounds__(256, 2) hop_mrhs_pipe_kernel(const HopArgs A, 
 // grid row, the loads of the next hop in flight through cp.async while the
 // present one is computed (FxStaged: 368 bytes of shared memory per thread,
 // which eight resident 64-thread blocks of 128 registers fill to 188 KB).
-// Bound by the issue of integer instructions (~7,300 per warp of sites, 1.9 per
+// Bound by the issue of integer instructions (~7,700 per warp of sites, 2.0 per
 // clock and SM; DRAM at half its rate), so several right-hand sides gain
 // nothing from sharing the links: a form with the links of a tile staged for
 // all of them took 1,727 us for the hopping term of 24^3 x 48 with 12
 // right-hand sides, one grid row per right-hand side 1,434 us.  32^3 x 64,
-// one right-hand side: 385 us, in FP64 arithmetic 1,628 us.  Reducing
-// launches use the full grid too; the partial sums are added by the last
-// block or (partials_only) by a finishing launch.
+// one right-hand side: 393 us (385 without the test for small components,
+// kFxLeast), in FP64 arithmetic 1,628 us.  Reducing launches use the full grid
+// too; the partial sums are added by the last block or (partials_only) by a
+// finishing launch.
 static constexpr int kFxBlock = 64;
 
 template <bool DAG, bool DOT, int CL>

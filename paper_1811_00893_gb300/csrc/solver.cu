@@ -328,9 +328,9 @@ int ensure_ws(wl_gauge g, int inner, int nrhs, int eo)
 {
     Workspace* w = g->ws;
     // Outer residual corrections of mixed-precision solves.  FP64 with
-    // fixed-point links (fx64.cuh): 32^3 x 64 hopping term 390 us, in df64
-    // (double-float) 455 us, and b and x need no second copy.  df64 for links that do not fit, and with a clover term,
-    // whose 6x6 products stay on the FP64 pipe.
+    // fixed-point links (fx64.cuh): 32^3 x 64 hopping term 393 us, in df64
+    // (double-float) 453 us, and b and x need no second copy.  df64 for links
+    // that do not fit, and with a clover term, whose 6x6 products stay on the FP64 pipe.
     const int outer = inner == WL_F64 || (g->fx64 && !g->has_clover) ? WL_F64 : WL_DF64;
     if (w && w->inner == inner && w->nrhs >= nrhs && w->eo == eo && w->outer == outer) return WL_OK;
     WL_CUDA(cudaDeviceSynchronize());
