@@ -28,7 +28,7 @@
 // ~16 dependent operations at 2^-53 of the partial sum.  What is small next to
 // 2^(e-1023) is computed in FP64 (kFxLeast).
 //
-// Links that do not fit (fx_link_fits in gauge.cu, at set-up: an entry above 1.25, or
+// Links that do not fit (fx_check_link in gauge.cu, at set-up: an entry above 1.25, or
 // rows or entries too small for multiples of 2^-59) keep plain FP64 for the whole lattice.
 //
 // Room: link entries have modulus <= 1.25, so |cross sum|
@@ -49,7 +49,7 @@ static constexpr double kFxMinLink = 0.125;             // least modulus of a ro
 static constexpr double kFxTinyLink = 0x1p-14;
 static constexpr int kFxTinyShare = 1024;
 
-// n_w as (wh, wl) of one real, |w| < 2: the 53-bit significand shifted to units of
+// n_w as (wh, wl) of one real: the 53-bit significand shifted to units of
 // 2^-59, rounded to nearest, ties to even.  Integer operations: with a multiplication
 // and a conversion per real on the FP64 pipe, the check's moduli there too and the link
 // in local memory, creating a gauge object of 32^3 x 64 in FP64 and FP32 took 6.1 ms, so
@@ -59,7 +59,7 @@ __device__ __forceinline__ void fx_split(double w, int& h, int& l)
     const unsigned long long b = (unsigned long long)__double_as_longlong(w);
     const int s = 1026 - ((int)(b >> 52) & 0x7ff);  // 3 for 1 <= |w| < 2
     long long n = 0;
-    if (s < 64) {  // (|w| >= 2^-60)
+    if (s > 0 && s < 64) {  // 2^-60 <= |w| < 8 (links with larger entries are not held so)
         const unsigned long long y = ((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10;
         n = (long long)((y + ((1ULL << (s - 1)) - 1) + (y >> s & 1)) >> s);
         if ((long long)b < 0) n = -n;
